@@ -20,7 +20,7 @@ LIB = os.path.join(OUT_DIR, "libgp_sscn.so")
 LIB_CHECK = os.path.join(OUT_DIR, "libgp_sscn_check.so")
 SOURCES = ["gp_api.cu", "gp_sweeps.cu", "gp_sweeps64.cu", "gp_reduce.cu", "gp_noalloc.cu",
            "gp_batch.cu"]
-HEADERS = ["gp_device.cuh", "gp_internal.h", "gp_arena.h"]
+HEADERS = ["gp_device.cuh", "gp_split.cuh", "gp_internal.h", "gp_arena.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 

@@ -99,6 +99,7 @@ struct Layout {
   size_t coef_off[2][3][2] = {};   // [mode][axis][A/B] byte offset from off_coef
   size_t fx_off[2] = {};           // trap factors along x per mode [pitch], from off_coef
   size_t fyz_off[2] = {};          // trap factor per row per mode, from off_coef
+  size_t ex_off[2] = {};           // FP64: the x factors less 1 in two FP32 parts, per mode
   size_t fxh_off[2] = {};          // the same for half a step (Strang splitting)
   size_t fyzh_off[2] = {};
   size_t npartials = 0;
@@ -205,6 +206,10 @@ const char* compute_layout(const gp_params* p, Layout* L) {
       (half ? L->fyzh_off : L->fyz_off)[m] = c;
       c = align_up(c + rows * L->rbytes * (m + 1), kAlign);
     }
+  for (int m = 0; m < 2 && L->rbytes == 8; ++m) {
+    L->ex_off[m] = c;
+    c = align_up(c + (size_t)L->pitch[m] * 8 * (m + 1), kAlign);
+  }
   off = align_up(off + c, kAlign);
   L->off_vtab = off;
   off = align_up(off + (size_t)(p->nx + p->ny + p->nz) * L->rbytes, kAlign);
@@ -487,6 +492,16 @@ void fill_sweep_params(gp_solver* s) {
       q.wait_ns = gpk::kWaitLimitNs;
       q.dV = p.dx * p.dy * p.dz;
       q.ntiles = s->L.ntiles_z[m];
+      if (s->line64 && (a < 2 || p.nz > 1)) {
+        // the increment form where the line qualifies (one norm partial per block)
+        const double h = a == 0 ? p.dx : a == 1 ? p.dy : p.dz, beta = p.dt / (4.0 * h * h);
+        q.inc_ex = coef + s->L.ex_off[m];
+        q.inc_amax = reinterpret_cast<int*>(s->step_ctr) + 1;
+        if (!gpk::inc64_setup(a, &q, m == 0 ? std::complex<double>(beta, 0.0)
+                                             : std::complex<double>(0.0, beta), m == 1) ||
+            (a == 2 && gpk::inc64_blocks(a, q, m == 1) > (long long)s->L.npartials))
+          q.inc_x = 0;
+      }
       q.trunc = s->trunc[m][a];
       if (q.trunc) {
         const int tiles32 = (p.nx + 31) / 32;
@@ -726,6 +741,19 @@ int upload_tables(gp_solver* s) {
       const double x = (i - 0.5 * (n[a] - 1)) * h[a];
       return 0.5 * w[a] * w[a] * x * x;
     };
+    // FP64: the x factors less 1 (expm1; cos - 1 = -2 sin^2 of half the angle) as FP32
+    // pairs: per 16-byte vector of a row the two high parts, then the two low ones
+    for (int i = 0; i < p.nx && f64; ++i) {
+      const double th = p.dt * pot(0, i), sn = std::sin(0.5 * th);
+      const double e[3] = {std::expm1(-th), -2.0 * sn * sn, -std::sin(th)};
+      for (int q = 0; q < 3; ++q) {
+        const float h = (float)e[q], l = (float)(e[q] - (double)h);
+        const size_t at = q == 0 ? L.ex_off[0] + (size_t)(i / 2) * 16 + (i % 2) * 4
+                                 : L.ex_off[1] + (size_t)i * 16 + (q - 1) * 4;
+        put<float>(buf, at, h);
+        put<float>(buf, at + 8, l);
+      }
+    }
     for (int half = 0; half < 2; ++half) {
       const double tau = half ? 0.5 * p.dt : p.dt;
       const size_t* fxo = half ? L.fxh_off : L.fx_off;
@@ -763,10 +791,12 @@ int set_scale_one(gp_solver* s) {
   return GP_OK;
 }
 
-// A new field: its imaginary-time steps (the FP32 factor's dither) count from zero, so
-// that the same field and the same steps give the same bits in any solver.
+// A new field: its imaginary-time steps (the FP32 factor's dither) count from zero, and
+// nothing is known of its largest value (the two words behind the count: the FP64
+// increment sweeps' noise floor), so that the same field and the same steps give the same
+// bits in any solver.
 int reset_steps(gp_solver* s) {
-  GP_CUDA(s, cudaMemsetAsync(s->step_ctr, 0, sizeof(unsigned int), s->stream));
+  GP_CUDA(s, cudaMemsetAsync(s->step_ctr, 0, 3 * sizeof(unsigned int), s->stream));
   return GP_OK;
 }
 
@@ -917,6 +947,8 @@ template <class R> int run_sweep(gp_solver* s, int axis) {
     e = gpk::launch_sweep_band_line(axis, q, m == 1, s->fast_grid[m][axis], s->stream);
   else if (q.trunc)
     e = gpk::launch_sweep_fast(axis, q, m == 1, s->fast_grid[m][axis], s->stream);
+  else if (s->line64 && q.inc_x)
+    e = gpk::launch_inc64(axis, q, m == 1, s->stream);
   else if (s->line64)
     e = gpk::launch_sweep64(axis, q, m == 1, s->stream);
   else if (axis == 0)

@@ -93,6 +93,16 @@ struct SweepParams {
   int band_cp;           // y / z: 1 = next turn's inputs copied to shared memory ahead (cp.async)
   int band_reg;          // x: 1 = the row in registers (k_sweep_x_reg)
   float band_dtg;        // x: dt g in FP32
+  // FP64 increment sweeps (gp_sweeps64.cu): decay factor rho of the CN solve's two
+  // one-sided recursions, rho + 1/rho = (1+2a)/a, in FP64 (re, im) and as the FP32 pairs
+  // (re hi, re lo, im hi, im lo); 16-byte vectors per block row and segments per line
+  int inc_x, inc_seg;    // inc_x = 0: not used
+  double rho[2];
+  float rho_f[4];
+  int inc_quiet;         // x: high word of |v| below which the nonlinear term is nothing
+  int* inc_amax;         // the field's largest |v| as an FP64 high word (see inc_floor)
+  const void* inc_ex;    // x: trap factor along x less 1, two-part FP32, per 16-byte vector of a row:
+                         // (h, h', l, l') of two real columns or of (re, im) of one complex
   // pointwise substep (x sweep only)
   int pw;                // 1: pointwise substep fused on load; 0: kinetic-only step
   const void* vx;
@@ -232,6 +242,12 @@ size_t x64_smem(bool complex_field);
 cudaError_t sweep64_prepare();
 long long sweep64_blocks(int axis, int nx, int ny, int nz);
 cudaError_t launch_sweep64(int axis, const SweepParams& p, bool complex_field, cudaStream_t st);
+// FP64 increment form of the sweeps: whether a line of n points with CN parameter
+// a (real: imaginary time, imaginary: real time) qualifies; fills p's inc_* and rho
+// fields (p.n, p.nx, p.ny, p.nz set); blocks of the launch, and the launch.
+bool inc64_setup(int axis, SweepParams* p, std::complex<double> a, bool complex_field);
+long long inc64_blocks(int axis, const SweepParams& p, bool complex_field);
+cudaError_t launch_inc64(int axis, const SweepParams& p, bool complex_field, cudaStream_t st);
 // Resident warps per SM of the streaming y / z kernel (occupancy calculator).
 int stream_warps_per_sm(int axis, bool complex_field, int trunc);
 

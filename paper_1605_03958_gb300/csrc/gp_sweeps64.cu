@@ -20,6 +20,11 @@
 // stored in place, then the back substitution), mostly through L2, in a fraction of
 // its arithmetic time.
 //
+// Lines of at least 16 points with |a| <= 1/32 (every configuration at dt <= h^2 / 8) take
+// the increment form instead (second half of this file), which moves all but one or two
+// FP64 operations per point to the FP32 pipe.  The kernels of this first half serve the
+// others: shorter lines, larger time steps.
+//
 //   x    a warp owns 32 consecutive rows, one row per lane.  Rows are contiguous, so a
 //        warp moves them through shared memory in chunks of C columns (32 real / 16
 //        complex, padded rows against bank conflicts): a chunk is loaded and stored
@@ -28,7 +33,12 @@
 //   y/z  a thread owns one line; lanes are consecutive x, so every access is coalesced.
 //        The line streams forward (forward values in place) and back, loads issued kU
 //        elements ahead.  z sums |u|^2 of its output for the renormalisation factor.
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+
 #include "gp_device.cuh"
+#include "gp_split.cuh"
 
 namespace gpk {
 
@@ -386,18 +396,574 @@ __global__ void __launch_bounds__(kLineThreads) k_sweep_line64(const __grid_cons
                                   p.status, p.dV);
 }
 
+// ------------------------------------------- sweeps y, z in increment form
+
+// The CN solve of a line as v plus an increment: with K the second difference (zero
+// ghosts), u = (I + aK)^{-1} (I - aK) v = v + 2a (I + aK)^{-1} s, s_j = v_{j-1} - 2 v_j +
+// v_{j+1}, and I + aK = (a / rho) (1 - rho S) (1 - rho S^{-1}) (S the shift), so
+//   y_j = s_j + rho y_{j-1},   z_j = y_j + rho z_{j+1},   u_j = v_j + 2 rho z_j.
+// z vanishes at the ghosts (it is odd about them): z_n = 0 starts the backward pass and
+// y_{-1} = -rho sum_k rho^k s_k the forward one.  |rho| <= 1/32 here (a <= 1/32), so the
+// recursions forget: a segment's carry-in is the 12-term tail (head) of its neighbour
+// (rho^12 < 2^-60), its far six terms in FP32 (rho^6 < 2^-29).
+//
+// What bounds it: FP64 arithmetic runs at 1/64 of FP32's rate here, so the increment is
+// formed in two-part FP32 (gp_split.cuh) and one DADD per point is left (14.7 us of FP64
+// pipe for 240 x 200 x 160 real points), against five FP64 operations per real point and
+// 18 per complex one in k_sweep_line64.  Measured at 240 x 200 x 160 (GB300, event-timed
+// launches): y 80 -> 44 us, z with its norm 106 -> 59 us; complex y 245 -> 91 us, z 290 ->
+// 83 us.  Now bound by issue (2.2-2.4 of 4 instructions per clock, 116 per real point,
+// 260 per complex one) and the FP64 pipe (34-54 %).  Accuracy: on smooth lines
+// s is exact and the increment's error is far below the final rounding (relative L2 of a
+// sweep against quadruple precision, a = 0.025: 4.8e-17, the rounding of u alone, where
+// the FP64 recurrence has 1.2e-16).  On a line of grid-scale noise s has no spare bits
+// left and two FP32 parts would lose to FP64 (4.2e-16), so a block that sees such values
+// (or any too large for FP32's range, or non-finite) evaluates its lines in FP64.
+//
+// A thread owns one 16-byte vector position (two real x or one complex x) and a segment of
+// 16 points of the line; the block holds whole lines (all segments of inc_x positions),
+// so the sweep works in place: every load precedes the first barrier, every store follows
+// it.  The segment's values arrive by cp.async (all in flight, no registers held) in
+// the thread's 16 shared-memory slots and the recursions work there in place; v is read
+// again, four points ahead, for the final addition.  (The segment in registers: 128 of
+// them, one block of 13 warps per SM, 68 us against 54 us for y.)  Blocks of about 128
+// threads: 96 and 192 measured slower over the three axes.
+constexpr int kIncL = 16;        // points per segment
+constexpr int kIncG = 4;         // values of v read ahead in the backward pass
+constexpr int kIncH = 12;        // terms of a carry
+constexpr int kIncNear = 6;      // of those, the near ones in two-part arithmetic
+constexpr int kIncThreads = 256; // most threads per block
+
+// Noise is looked for in values above 2^-10 of the field's largest (noise below that, in
+// the far tails, adds nothing to the field's error).  The x sweep takes the largest FP64 high
+// word (as an integer, so the order of the blocks does not matter) into amax[0]; the y
+// sweep uses it and copies it to amax[1], which the z sweep and the next x sweep use; the
+// z sweep clears amax[0].  Zero (a new field, no x sweep of this form): no floor.
+__device__ __forceinline__ float inc_floor(const int* amax) {
+  const int t = addmax0(*amax, -kSplitOff);
+  return t >= kSplitTooBig ? 0.f : bits_f((uint32_t)t << 3) * 0x1p-10f;
+}
+
+template <bool CPLX> struct IncRho;
+template <> struct IncRho<false> {
+  Coef r;
+  double d;
+  __device__ explicit IncRho(const SweepParams& p)
+      : r(coef_pair(f2(p.rho_f[0]), f2(p.rho_f[1]))), d(p.rho[0]) {}
+  __device__ __forceinline__ Prod mul(const Two& x) const { return two_mul(r, x); }
+  __device__ __forceinline__ float2 mul_add(float2 x, float2 s) const { return fma2(r.h, x, s); }
+  __device__ __forceinline__ double2 mul_add(double2 x, double2 s) const {
+    return make_double2(fma(d, x.x, s.x), fma(d, x.y, s.y));
+  }
+};
+template <> struct IncRho<true> {
+  Coef r, i;   // i holds (-im, im): it multiplies (im, re)
+  double2 d;
+  __device__ explicit IncRho(const SweepParams& p)
+      : r(coef_pair(f2(p.rho_f[0]), f2(p.rho_f[1]))),
+        i(coef_pair(f2(-p.rho_f[2], p.rho_f[2]), f2(-p.rho_f[3], p.rho_f[3]))),
+        d(make_double2(p.rho[0], p.rho[1])) {}
+  __device__ __forceinline__ Prod mul(const Two& x) const {
+    Two sw;
+    sw.h = f2(x.h.y, x.h.x);
+    sw.l = f2(x.l.y, x.l.x);
+    return prod_add(two_mul(i, sw), two_mul(r, x));
+  }
+  __device__ __forceinline__ float2 mul_add(float2 x, float2 s) const {
+    return fma2(i.h, f2(x.y, x.x), fma2(r.h, x, s));
+  }
+  __device__ __forceinline__ double2 mul_add(double2 x, double2 s) const { return cfma(d, x, s); }
+};
+
+// The 12-term carry sum_k rho^k at(k).
+template <class RHO, class AT> __device__ __forceinline__ Two inc_carry(const RHO& rho, AT at) {
+  float2 t = at(kIncH - 1).h;
+#pragma unroll
+  for (int k = kIncH - 2; k >= kIncNear; --k) t = rho.mul_add(t, at(k).h);
+  Two w;
+  w.h = t;
+  w.l = f2(0.f);
+#pragma unroll
+  for (int k = kIncNear - 1; k >= 0; --k) w = two_add(at(k), rho.mul(w));
+  return w;
+}
+template <class RHO, class AT> __device__ __forceinline__ double2 inc_carry64(const RHO& rho, AT at) {
+  double2 t = at(kIncH - 1);
+  for (int k = kIncH - 2; k >= 0; --k) t = rho.mul_add(t, at(k));
+  return t;
+}
+
+__device__ __forceinline__ void put_two(float4* q, const Two& w) {
+  *q = make_float4(w.h.x, w.h.y, w.l.x, w.l.y);
+}
+__device__ __forceinline__ Two get_two(const float4* q) {
+  const float4 f = *q;
+  return two_scalar(f2(f.x, f.y), f2(f.z, f.w));
+}
+__device__ __forceinline__ void put_d2(float4* q, double2 w) { *reinterpret_cast<double2*>(q) = w; }
+__device__ __forceinline__ double2 get_d2(const float4* q) { return *reinterpret_cast<const double2*>(q); }
+
+// One thread's segment [j0, j0 + kIncL) of a line of n points: slot[u TS] holds its v
+// (zero from n on) and is overwritten; carry (and carry + T) are its exchange places, the
+// neighbouring segments' lie X threads away; before / after: the values at j0 - 1 and
+// j0 + kIncL (zero outside the line).  io.load(u): v again for the final addition;
+// io.store(u, v, c): the increment c of point j0 + u (j0 + u < n); io.rd(j): v of any point
+// of the line (FP64 path).  Every thread of the block must call it; `on`: the thread owns a
+// segment.
+template <bool CPLX, class IO>
+__device__ __forceinline__ void inc_segment(const IncRho<CPLX>& rho, float4* slot, int TS, float4* carry,
+                                            int T, int X, int sg, int nseg, int j0, int n, bool on,
+                                            double2 before, double2 after, float least, IO& io) {
+  int tmax = 0;
+  // noise: somewhere sampled, the second difference is opposite in sign to v and larger
+  // than the values (complex: the moduli) around it and than least
+  bool fp64 = false;
+  {
+    const double2 v0 = get_d2(slot);
+    Three a = split3(before.x, before.y, &tmax), b = split3(v0.x, v0.y, &tmax);
+#pragma unroll 8
+    for (int u = 0; u < kIncL; ++u) {
+      const double2 vn = u + 1 < kIncL ? get_d2(slot + (u + 1) * TS) : after;
+      const Three c = split3(vn.x, vn.y, &tmax);
+      const Two s = second_difference(a, b, c);
+      put_two(slot + u * TS, s);
+      if (u % 4 == 2) {
+        float lx = fmaxf(least, fmaxf(fabsf(a.h.x), fmaxf(fabsf(b.h.x), fabsf(c.h.x))));
+        float ly = fmaxf(least, fmaxf(fabsf(a.h.y), fmaxf(fabsf(b.h.y), fabsf(c.h.y))));
+        if (CPLX) lx = ly = fmaxf(lx, ly);
+        fp64 = fp64 || (fabsf(s.h.x) > lx && s.h.x * b.h.x < 0.f) ||
+               (fabsf(s.h.y) > ly && s.h.y * b.h.y < 0.f);
+      }
+      a = b;
+      b = c;
+    }
+  }
+  fp64 = fp64 || tmax >= kSplitTooBig;
+  if (!__syncthreads_or(on && fp64)) {
+    // carry out to the next segment: the tail of s; the first segment also starts itself
+    put_two(carry, inc_carry(rho, [&](int k) { return get_two(slot + (kIncL - 1 - k) * TS); }));
+    Prod pr = prod_zero();
+    if (sg == 0)
+      pr = rho.mul(two_neg(prod_two(rho.mul(inc_carry(rho, [&](int k) { return get_two(slot + k * TS); })))));
+    __syncthreads();
+    if (sg > 0) pr = rho.mul(get_two(carry - X));
+#pragma unroll 4
+    for (int u = 0; u < kIncL; ++u) {
+      const Two y = j0 + u < n ? two_add(get_two(slot + u * TS), pr) : two_zero();
+      put_two(slot + u * TS, y);
+      pr = rho.mul(y);
+    }
+    put_two(carry + T, inc_carry(rho, [&](int k) { return get_two(slot + k * TS); }));
+    double2 v[kIncG];   // v again, the last group
+#pragma unroll
+    for (int q = 0; q < kIncG; ++q) v[q] = io.load(kIncL - kIncG + q);
+    __syncthreads();
+    pr = prod_zero();
+    if (on && sg + 1 < nseg) pr = rho.mul(get_two(carry + T + X));
+    for (int g = kIncL - kIncG; g >= 0; g -= kIncG) {
+      double2 nxt[kIncG];   // the group below, in flight while this one is computed
+#pragma unroll
+      for (int q = 0; q < kIncG; ++q) nxt[q] = g > 0 ? io.load(g - kIncG + q) : v[q];
+#pragma unroll
+      for (int q = kIncG - 1; q >= 0; --q) {
+        const int u = g + q;
+        pr = rho.mul(two_add(get_two(slot + u * TS), pr));
+        const Two c = two_norm(pr);
+        const double2 cd = make_double2(to_double(c.h.x, c.l.x, 1), to_double(c.h.y, c.l.y, 1));
+        if (on && j0 + u < n) io.store(u, v[q], cd);
+      }
+#pragma unroll
+      for (int q = 0; q < kIncG; ++q) v[q] = nxt[q];
+    }
+  } else {
+    // the same recursions in FP64
+    {
+      double2 a = before, b = io.rd(j0);
+      for (int u = 0; u < kIncL; ++u) {
+        const double2 c = io.rd(j0 + u + 1);
+        put_d2(slot + u * TS, make_double2((c.x - b.x) - (b.x - a.x), (c.y - b.y) - (b.y - a.y)));
+        a = b;
+        b = c;
+      }
+    }
+    const double2 zero = make_double2(0.0, 0.0);
+    put_d2(carry, inc_carry64(rho, [&](int k) { return get_d2(slot + (kIncL - 1 - k) * TS); }));
+    double2 prev = zero;
+    if (sg == 0) {
+      const double2 t = rho.mul_add(inc_carry64(rho, [&](int k) { return get_d2(slot + k * TS); }), zero);
+      prev = make_double2(-t.x, -t.y);
+    }
+    __syncthreads();
+    if (sg > 0) prev = get_d2(carry - X);
+    for (int u = 0; u < kIncL; ++u) {
+      prev = j0 + u < n ? rho.mul_add(prev, get_d2(slot + u * TS)) : zero;
+      put_d2(slot + u * TS, prev);
+    }
+    put_d2(carry + T, inc_carry64(rho, [&](int k) { return get_d2(slot + k * TS); }));
+    __syncthreads();
+    double2 z = zero;
+    if (on && sg + 1 < nseg) z = get_d2(carry + T + X);
+    for (int u = kIncL - 1; u >= 0; --u) {
+      z = rho.mul_add(z, get_d2(slot + u * TS));
+      const double2 v = io.load(u), c = rho.mul_add(z, zero);
+      if (on && j0 + u < n) io.store(u, v, make_double2(2.0 * c.x, 2.0 * c.y));
+    }
+  }
+}
+
+template <bool CPLX, int AXIS, bool NORM>
+__global__ void __launch_bounds__(kIncThreads) k_sweep_inc64(const __grid_constant__ SweepParams p) {
+  extern __shared__ __align__(16) float4 inc_smem[];
+  const int X = p.inc_x, nseg = p.inc_seg, n = p.n;
+  const int tid = threadIdx.x, T = blockDim.x;
+  float4* slot = inc_smem + tid;               // [kIncL][T]: v, then s, then y (two-part or FP64)
+  float4* carry = inc_smem + kIncL * T + tid;  // [2][T]: tails of s, heads of y
+  pdl_begin();
+  const int sg = tid / X, xl = tid - sg * X;
+  const int nvec = CPLX ? p.nx : (p.nx + 1) / 2;
+  const int ntile = (nvec + X - 1) / X;
+  const int o = blockIdx.x / ntile, xv = (blockIdx.x - o * ntile) * X + xl;
+  const size_t P = (size_t)(CPLX ? p.pitch : p.pitch / 2);   // row pitch in vectors
+  const int j0 = sg * kIncL;
+  struct IO {
+    double2* line;
+    size_t stride;
+    int j0, n;
+    bool on;
+    double acc;
+    long long first, nall;   // bounds checks
+    int* status;
+    __device__ bool inside(int j) const {
+      return on && j >= 0 && j < n && GP_IN(first + (long long)j * (long long)stride, nall, status);
+    }
+    __device__ double2 rd(int j) const { return inside(j) ? line[(size_t)j * stride] : make_double2(0.0, 0.0); }
+    __device__ double2 load(int u) const { return rd(j0 + u); }
+    __device__ void store(int u, double2 v, double2 c) {
+      const double2 w = make_double2(v.x + c.x, v.y + c.y);
+      if (!GP_IN(first + (long long)(j0 + u) * (long long)stride, nall, status)) return;
+      line[(size_t)(j0 + u) * stride] = w;
+      if constexpr (NORM) acc = fma(w.x, w.x, fma(w.y, w.y, acc));
+    }
+  } io;
+  io.on = sg < nseg && xv < nvec;
+  io.stride = AXIS == 1 ? P : P * (size_t)p.ny;
+  io.first = (long long)((AXIS == 1 ? (size_t)o * P * p.ny : (size_t)o * P) + (io.on ? xv : 0));
+  io.nall = (long long)P * p.ny * p.nz;   // vectors of the field
+  io.line = reinterpret_cast<double2*>(p.psi) + io.first;
+  io.j0 = j0;
+  io.n = n;
+  io.acc = 0.0;
+  io.status = p.status;
+#pragma unroll
+  for (int u = 0; u < kIncL; ++u) {
+    const bool ok = io.inside(j0 + u);
+    cp_async16_zfill(slot + u * T, io.line + (ok ? (size_t)(j0 + u) * io.stride : 0), ok);
+  }
+  cp_async_commit();
+  const double2 before = io.rd(j0 - 1), after = io.rd(j0 + kIncL);
+  const IncRho<CPLX> rho(p);
+  const float least = inc_floor(p.inc_amax + (AXIS == 1 ? 0 : 1));
+  if (blockIdx.x == 0 && tid == 0) {
+    if (AXIS == 1) p.inc_amax[1] = p.inc_amax[0];
+    else p.inc_amax[0] = 0;
+  }
+  cp_async_wait<0>();
+  inc_segment<CPLX>(rho, slot, T, carry, T, X, sg, nseg, j0, n, io.on, before, after, least, io);
+  if constexpr (NORM) norm_finish(io.acc, p.partials, p.counter, gridDim.x, blockIdx.x, p.scale_out,
+                                  p.status, p.dV);
+}
+
+// ---------------------------------------------- sweep x in increment form
+
+// The pending factor and the pointwise substep as an increment too: with f the trap
+// factor, e = s f exp(-y) - 1 (real; complex: s f cis(-y) - 1), y = dt g s^2 |v|^2,
+//   e = E + (1 + E) q,   E = ex + er + ex er,   q = exp(-y) - 1 (cis(-y) - 1),
+// ex the column's factor less 1 (two-part table, from expm1 / sin^2 in FP64), er the
+// row's times the pending factor, less 1; v' = v + v e: real, e as FP64 and one DFMA; complex,
+// v e in two-part FP32 and one DADD per part.  q is skipped where every lane of the warp has |y| < 2^-56, and taken from short or
+// long Taylor sums by the size of y; a warp with |y| > 1/8, |E| > 1/4 (where 1 + E in two
+// parts would lose to FP64) or values out of range computes the substep in FP64.
+// Measured at 240 x 200 x 160 with the solve: 284 us (k_sweep_x64 at its shortest
+// polynomial; 620 us where the density calls for the longer one) -> 92 us, complex 686
+// -> 194 us.
+//
+// A block owns inc_x row vectors (real: pairs of rows; complex: rows) and works in three
+// passes: lanes along the rows (coalesced) for the substep, v' to the field and to the
+// segments' slots in shared memory; one segment of 16 columns per thread for the solve
+// (as the y / z kernel; the increments replace the slots); lanes along the rows again
+// for u = v' + c.
+constexpr float kIncBigE = 0.25f;
+
+// v' in FP64 (f: the folded factor times the trap factors; real, complex)
+__device__ __forceinline__ double pointwise64(double v, double f, double cy) {
+  const double y = cy * (v * v);
+  const unsigned long long mb = abs_bits(y);
+  double q;
+  if (mb <= kBits2m10) {
+    q = fma(y, fma(y, fma(y, fma(y, kSignedInvFact[4], kSignedInvFact[3]), 0.5), -1.0), 1.0);
+  } else if (mb <= kBits2m4) {
+    q = fma(y, kSignedInvFact[9], kSignedInvFact[8]);
+#pragma unroll
+    for (int k = 7; k >= 0; --k) q = fma(y, q, kSignedInvFact[k]);
+  } else {
+    q = exp(-y);
+  }
+  return v * f * q;
+}
+
+__device__ __forceinline__ double2 pointwise64(double2 v, double2 f, double cy) {
+  const double th = cy * fma(v.x, v.x, v.y * v.y);
+  const unsigned long long mb = abs_bits(th);
+  double cs, sn;
+  if (mb <= kBits2m8) {
+    const double t2 = th * th;
+    cs = fma(t2, fma(t2, 1.0 / 24.0, -0.5), 1.0);
+    sn = th * fma(t2, fma(t2, 1.0 / 120.0, -1.0 / 6.0), 1.0);
+  } else {
+    sincos(th, &sn, &cs);
+  }
+  return cmul(cmul(v, f), make_double2(cs, -sn));
+}
+
+template <bool CPLX>
+__global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_constant__ SweepParams p) {
+  extern __shared__ __align__(16) float4 inc_smem[];
+  const int X = p.inc_x, nseg = p.inc_seg, nx = p.nx;
+  const int tid = threadIdx.x, T = blockDim.x, TS = T + 1;   // one slot of padding: see `place`
+  constexpr int RPV = CPLX ? 1 : 2;                          // rows per row vector
+  const int rows_t = X * RPV;
+  float4* slots = inc_smem;                                  // [kIncL][TS]
+  float4* carry = inc_smem + kIncL * TS + tid;               // [2][T]
+  float4* rowc = inc_smem + kIncL * TS + 2 * T;              // per tile row: the row's factor
+  const long long nrows = (long long)p.ny * p.nz;
+  const long long r0 = (long long)blockIdx.x * rows_t;
+  const int rows = (int)min((long long)rows_t, nrows - r0);
+  const int P = CPLX ? p.pitch : p.pitch / 2, nvec = CPLX ? nx : (nx + 1) / 2;   // vectors per row
+  double2* field = reinterpret_cast<double2*>(p.psi) + (size_t)r0 * P;
+  const long long nall = nrows * P, at0 = r0 * P;            // bounds checks
+  (void)nall;
+  (void)at0;
+  __shared__ double head_d[3];   // the factor applied ahead, the one folded in, dt g s^2
+  __shared__ int head_max;
+  const IncRho<CPLX> rho(p);
+  pdl_begin();
+  // FP64 is slow even a few operations per thread: one thread forms the block's scalars
+  if (tid == 0) {
+    const double s = *p.scale;
+    // folded into the rows' increments unless it is far from 1 (or not a number)
+    const bool fold = fabs(s - 1.0) <= 0.0625;
+    head_d[0] = fold ? 1.0 : s;
+    head_d[1] = fold ? s : 1.0;
+    head_d[2] = p.dt * p.g * head_d[1] * head_d[1];
+    head_max = 0;
+  }
+  const float least = inc_floor(p.inc_amax + 1);
+  __syncthreads();
+  const double spre = head_d[0], s = head_d[1], cy = head_d[2];
+  const bool pre = __double2hiint(spre) != 0x3ff00000 || __double2loint(spre) != 0;
+  const bool pw = p.pw != 0;
+  const bool work = pw || __double2hiint(s) != 0x3ff00000 || __double2loint(s) != 0;
+  // rows' factors f = s (trap factor) and er = f - 1: real (f, f', er, er'); complex
+  // f, f with its parts exchanged, er, each (re, im, re', im')
+  for (int r = tid; r < rows; r += T) {
+    if constexpr (!CPLX) {
+      const double f0 = pw ? static_cast<const double*>(p.band_fyz)[r0 + r] : 1.0;
+      const double f = f0 * s, e = fma(f0, s, -1.0);
+      const float fh = (float)f, eh = (float)e;
+      rowc[r] = make_float4(fh, (float)(f - (double)fh), eh, (float)(e - (double)eh));
+    } else {
+      const double2 f0 = pw ? static_cast<const double2*>(p.band_fyz)[r0 + r] : make_double2(1.0, 0.0);
+      const double fr = f0.x * s, fi = f0.y * s, er = fma(f0.x, s, -1.0);
+      const float rh = (float)fr, ih = (float)fi, eh = (float)er;
+      const float rl = (float)(fr - (double)rh), il = (float)(fi - (double)ih);
+      rowc[3 * r] = make_float4(rh, ih, rl, il);
+      rowc[3 * r + 1] = make_float4(ih, rh, il, rl);
+      rowc[3 * r + 2] = make_float4(eh, ih, (float)(er - (double)eh), il);
+    }
+  }
+  __syncthreads();
+  const Coef cyc = coef_pair(f2((float)cy), f2((float)(cy - (double)(float)cy)));
+  int vmax = 0;
+  // In the two passes along the rows a thread keeps to one vector position (column) per
+  // chunk of `per` positions and walks down the tile, `grp` rows at a time.  Column c of
+  // row r lies in the slot of segment c / 16, point c mod 16, row vector r / RPV; points
+  // are TS slots apart, so that lanes on consecutive columns spread over the banks.
+  const int nchunk = (nvec + T - 1) / T, per = (nvec + nchunk - 1) / nchunk, grp = T / per;
+  const int ro = tid / per, co = tid - ro * per;
+  const int rounds = (rows_t + grp - 1) / grp;
+  auto place = [&](int cv) {   // of row 0; row r is 16 / RPV bytes times r further
+    const int c = CPLX ? cv : 2 * cv;
+    return reinterpret_cast<double*>(slots + (c % kIncL) * TS + (c / kIncL) * X);
+  };
+  for (int ch = 0; ch < nchunk; ++ch) {
+    const int cv = ch * per + co;
+    const bool con = ro < grp && cv < nvec;
+    float4 ext = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (pw && con) ext = __ldg(static_cast<const float4*>(p.inc_ex) + cv);
+    // the column's factor as the constant of the products with the rows' factors
+    const Coef ex = CPLX ? coef_pair(f2(ext.x), f2(ext.z)) : coef_pair(f2(ext.x, ext.y), f2(ext.z, ext.w));
+    const Coef exi = coef_pair(f2(-ext.y, ext.y), f2(-ext.w, ext.w));
+    double* dst = place(con ? cv : 0);
+    const double2 zero = make_double2(0.0, 0.0);
+    auto fetch = [&](int r) {
+      return con && r < rows && GP_IN(at0 + (long long)r * P + cv, nall, p.status)
+                 ? field[(size_t)r * P + cv] : zero;
+    };
+    double2 nxt = fetch(ro);
+    for (int q = 0; q < rounds; ++q) {   // (full rounds: every lane takes part in the votes)
+      const int r = ro + q * grp;
+      const bool live = con && r < rows;
+      double2 v = nxt;
+      if (q + 1 < rounds) nxt = fetch(r + grp);
+      if (pre) {
+        v.x *= spre;
+        v.y *= spre;
+      }
+      const int vm = imax(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
+      vmax = imax(vmax, vm);
+      if (work) {
+        const float4* rc = rowc + (CPLX ? 3 : 1) * (live ? r : 0);
+        Two e;
+        if constexpr (!CPLX) {
+          const float4 f = rc[0];
+          e = two_add(two_scalar(f2(f.z), f2(f.w)), two_mul(ex, two_scalar(f2(f.x), f2(f.y))));
+        } else {
+          e = two_add(get_two(rc + 2), prod_add(two_mul(exi, get_two(rc + 1)), two_mul(ex, get_two(rc))));
+        }
+        bool ok = fmaxf(fabsf(e.h.x), fabsf(e.h.y)) <= kIncBigE;
+        int tmax = 0;
+        Two V;
+        if (CPLX) {
+          V = split2(v.x, v.y, &tmax);
+          ok = ok && tmax < kSplitTooBig;
+        }
+        if (pw && !__all_sync(0xffffffffu, vm < p.inc_quiet)) {
+          if (!CPLX) V = split2(v.x, v.y, &tmax);
+          // y = cy |v|^2 in natural scale
+          const Two h = two_scalar(mul2(V.h, f2(0x1p-56f)), mul2(V.l, f2(0x1p-56f)));
+          Two d = two_mul(h, h);
+          if (CPLX) d = two_add(d, two_swap(d));   // re^2 + im^2 in both lanes
+          Two y = prod_two(two_mul(cyc, d));
+          const float ym = fmaxf(fabsf(y.h.x), fabsf(y.h.y));
+          ok = ok && ym <= 0.125f && tmax < kSplitTooBig;
+          Two qv;
+          if (__all_sync(0xffffffffu, ym <= 0x1p-10f || !ok)) {
+            qv = CPLX ? two_cis_neg_m1_small(y) : two_expm1_neg_small(y);
+          } else {
+            const int halvings = __all_sync(0xffffffffu, ym <= (CPLX ? 0.0625f : 0.03125f) || !ok) ? 0
+                                 : __all_sync(0xffffffffu, ym <= (CPLX ? 0.125f : 0.0625f) || !ok) ? 1 : 2;
+            const float sc = halvings == 0 ? 1.f : halvings == 1 ? 0.5f : 0.25f;
+            y = two_scalar(mul2(y.h, f2(sc)), mul2(y.l, f2(sc)));
+            qv = CPLX ? two_cis_neg_m1(y) : two_expm1_neg(y);
+            for (int k = 0; k < halvings; ++k)
+              qv = two_add(two_scalar(add2(qv.h, qv.h), add2(qv.l, qv.l)), CPLX ? two_cmul(qv, qv) : two_mul(qv, qv));
+          }
+          e = two_add(two_add(e, qv), CPLX ? two_cmul(e, qv) : two_mul(e, qv));
+        }
+        if (__all_sync(0xffffffffu, ok || !live)) {
+          if constexpr (CPLX) {
+            const Two c = two_norm(two_cmul(V, e));
+            v.x += to_double(c.h.x, c.l.x, 0);
+            v.y += to_double(c.h.y, c.l.y, 0);
+          } else {
+            const Two c = two_norm(e);
+            v.x = fma(v.x, to_double(c.h.x, c.l.x, kSplitShift), v.x);
+            v.y = fma(v.y, to_double(c.h.y, c.l.y, kSplitShift), v.y);
+          }
+        } else if (live) {
+          const double c2 = pw ? cy : 0.0;
+          if constexpr (!CPLX) {
+            const double fr = pw ? s * static_cast<const double*>(p.band_fyz)[r0 + r] : s;
+            const double* fx = static_cast<const double*>(p.band_fx);
+            v.x = pointwise64(v.x, pw ? fr * fx[2 * cv] : fr, c2);
+            v.y = pointwise64(v.y, pw ? fr * fx[2 * cv + 1] : fr, c2);
+          } else {
+            const double2 rf = pw ? static_cast<const double2*>(p.band_fyz)[r0 + r] : make_double2(1.0, 0.0);
+            const double2 f = pw ? static_cast<const double2*>(p.band_fx)[cv] : make_double2(1.0, 0.0);
+            v = pointwise64(v, cmul(make_double2(s * f.x, s * f.y), rf), c2);
+          }
+        }
+      }
+      if (live && (work || pre) && GP_IN(at0 + (long long)r * P + cv, nall, p.status))
+        field[(size_t)r * P + cv] = v;
+      if (con && r < rows_t) {
+        if constexpr (CPLX) {
+          *reinterpret_cast<double2*>(dst + 2 * r) = v;
+        } else {
+          dst[r] = v.x;
+          dst[r + 2 * TS] = v.y;
+        }
+      }
+    }
+  }
+  vmax = __reduce_max_sync(0xffffffffu, vmax);
+  if ((tid & 31) == 0) atomicMax(&head_max, vmax);
+  __syncthreads();
+  if (tid == 0) atomicMax(p.inc_amax, head_max);
+  {
+    const int sg = tid / X, xl = tid - sg * X;
+    const int j0 = sg * kIncL;
+    struct IO {
+      float4* slot;
+      const double* row[2];   // v' of the thread's row(s) in the field
+      int TS, j0, nx;
+      bool on;
+      __device__ double2 rd(int j) const {
+        if (!on || j < 0 || j >= nx) return make_double2(0.0, 0.0);
+        if constexpr (CPLX) return reinterpret_cast<const double2*>(row[0])[j];
+        return make_double2(row[0][j], row[1] ? row[1][j] : 0.0);
+      }
+      __device__ double2 load(int) const { return make_double2(0.0, 0.0); }
+      __device__ void store(int u, double2, double2 c) { put_d2(slot + u * TS, c); }
+    } io;
+    io.on = sg < nseg && xl * RPV < rows;
+    io.slot = slots + tid;
+    io.TS = TS;
+    io.j0 = j0;
+    io.nx = nx;
+    io.row[0] = reinterpret_cast<const double*>(field + (size_t)(xl * RPV) * P);
+    io.row[1] = !CPLX && xl * RPV + 1 < rows ? reinterpret_cast<const double*>(field + (size_t)(xl * RPV + 1) * P)
+                                             : nullptr;
+    // columns past the row read as zero
+    for (int u = max(0, (CPLX ? nx : 2 * nvec) - j0); u < kIncL; ++u)
+      if (tid < X * nseg) put_d2(slots + tid + u * TS, make_double2(0.0, 0.0));
+    double2 before = make_double2(0.0, 0.0), after = before;
+    if (io.on && sg > 0) before = get_d2(slots + tid - X + (kIncL - 1) * TS);
+    if (io.on && sg + 1 < nseg) after = get_d2(slots + tid + X);
+    __syncthreads();
+    inc_segment<CPLX>(rho, slots + tid, TS, carry, T, X, sg, nseg, j0, nx, io.on, before, after, least, io);
+  }
+  __syncthreads();
+  for (int ch = 0; ch < nchunk; ++ch) {
+    const int cv = ch * per + co;
+    if (ro >= grp || cv >= nvec) continue;
+    const double* src = place(cv);
+    const bool pad = !CPLX && 2 * cv + 1 >= nx;
+#pragma unroll 4
+    for (int r = ro; r < rows; r += grp) {
+      if (!GP_IN(at0 + (long long)r * P + cv, nall, p.status)) continue;
+      const double2 v = field[(size_t)r * P + cv];
+      const double2 c = CPLX ? *reinterpret_cast<const double2*>(src + 2 * r)
+                             : make_double2(src[r], pad ? 0.0 : src[r + 2 * TS]);
+      field[(size_t)r * P + cv] = make_double2(v.x + c.x, v.y + c.y);
+    }
+  }
+}
+
 // ------------------------------------------------------------------ launchers
 
 size_t x64_smem(bool complex_field) {
   return complex_field ? X64Geom<true>::smem : X64Geom<false>::smem;
 }
 
+static cudaError_t inc64_prepare();
 cudaError_t sweep64_prepare() {
   cudaError_t e = cudaFuncSetAttribute(k_sweep_x64<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)X64Geom<false>::smem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_sweep_x64<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)X64Geom<true>::smem);
+  if (e == cudaSuccess) e = inc64_prepare();
   return e;
 }
 
@@ -432,6 +998,97 @@ cudaError_t launch_sweep64(int axis, const SweepParams& p, bool complex_field, c
   // the norm is summed in imaginary time only (real field)
   return complex_field ? cudaLaunchKernelEx(&cfg, k_sweep_line64<true, 2, false>, p)
                        : cudaLaunchKernelEx(&cfg, k_sweep_line64<false, 2, true>, p);
+}
+
+// Lines of at least 16 points (a carry's 12 terms lie within a segment and its line) and
+// a <= 1/32 (rho^12 < 2^-60).  Positions per block: enough for about 256 threads on short
+// lines, fewer on long ones so that a block keeps to kIncThreads; whole tiles of nearly
+// equal width.
+bool inc64_setup(int axis, SweepParams* p, std::complex<double> a, bool complex_field) {
+  p->inc_x = 0;
+  if (p->n < 16 || std::abs(a) > 1.0 / 32) return false;
+  // block rows: 16-byte vectors along x (y, z sweeps) or pairs of rows / rows (x sweep)
+  const long long nrows = (long long)p->ny * p->nz;
+  const int nvec = axis == 0 ? (int)(complex_field ? nrows : (nrows + 1) / 2)
+                             : complex_field ? p->nx : (p->nx + 1) / 2;
+  const int nseg = (p->n + kIncL - 1) / kIncL;
+  const int most = std::max(1, std::min(kIncThreads / nseg, std::max(axis == 0 ? 4 : 8, 128 / nseg)));
+  const int tiles = (nvec + most - 1) / most;
+  p->inc_seg = nseg;
+  p->inc_x = (nvec + tiles - 1) / tiles;
+  const std::complex<double> r = 2.0 * a / (1.0 + 2.0 * a + std::sqrt(1.0 + 4.0 * a));
+  const double part[2] = {r.real(), r.imag()};
+  for (int q = 0; q < 2; ++q) {
+    p->rho[q] = part[q];
+    p->rho_f[2 * q] = (float)part[q];
+    p->rho_f[2 * q + 1] = (float)(part[q] - (double)p->rho_f[2 * q]);
+  }
+  return true;
+}
+
+// x: slots with one of padding per point, carries, the rows' factors (real: two rows of one
+// float4 per row vector; complex: one row of three)
+static size_t inc64_x_smem(unsigned threads, int X) {
+  return ((size_t)kIncL * (threads + 1) + 2 * threads + 3 * X) * sizeof(float4);
+}
+
+// shared-memory limit of the increment kernels (blocks of kIncThreads)
+static cudaError_t inc64_prepare() {
+  void (*const k[4])(SweepParams) = {k_sweep_inc64<false, 1, false>, k_sweep_inc64<false, 2, true>,
+                                     k_sweep_inc64<true, 1, false>, k_sweep_inc64<true, 2, false>};
+  for (auto f : k) {
+    const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)((kIncL + 2) * kIncThreads * sizeof(float4)));
+    if (e != cudaSuccess) return e;
+  }
+  void (*const kx[2])(SweepParams) = {k_sweep_xinc64<false>, k_sweep_xinc64<true>};
+  for (auto f : kx) {
+    const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)inc64_x_smem(kIncThreads, kIncThreads));
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+long long inc64_blocks(int axis, const SweepParams& p, bool complex_field) {
+  if (axis == 0) {
+    const long long rows = (long long)p.inc_x * (complex_field ? 1 : 2);
+    return ((long long)p.ny * p.nz + rows - 1) / rows;
+  }
+  const int nvec = complex_field ? p.nx : (p.nx + 1) / 2;
+  return (long long)((nvec + p.inc_x - 1) / p.inc_x) * (axis == 1 ? p.nz : p.ny);
+}
+
+cudaError_t launch_inc64(int axis, const SweepParams& p, bool complex_field, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cfg.stream = st;
+  cfg.gridDim = dim3((unsigned)inc64_blocks(axis, p, complex_field));
+  cfg.blockDim = dim3((unsigned)((p.inc_x * p.inc_seg + 31) / 32 * 32));
+  cfg.dynamicSmemBytes = (size_t)(kIncL + 2) * cfg.blockDim.x * sizeof(float4);
+  if (axis == 0) {
+    cfg.dynamicSmemBytes = inc64_x_smem(cfg.blockDim.x, p.inc_x);
+    // high word of the |v| below which |y| < 2^-56 (complex: each part), the folded factor
+    // being at most 1.0625
+    SweepParams q = p;
+    const double most = 0x1p-56 / (1.13 * p.dt * std::fabs(p.g));
+    double lim = std::sqrt(complex_field ? 0.5 * most : most);
+    if (!(lim < 1e200)) lim = 1e200;   // g = 0
+    uint64_t w;
+    std::memcpy(&w, &lim, 8);
+    q.inc_quiet = (int)(w >> 32);
+    return complex_field ? cudaLaunchKernelEx(&cfg, k_sweep_xinc64<true>, q)
+                         : cudaLaunchKernelEx(&cfg, k_sweep_xinc64<false>, q);
+  }
+  if (axis == 1)
+    return complex_field ? cudaLaunchKernelEx(&cfg, k_sweep_inc64<true, 1, false>, p)
+                         : cudaLaunchKernelEx(&cfg, k_sweep_inc64<false, 1, false>, p);
+  return complex_field ? cudaLaunchKernelEx(&cfg, k_sweep_inc64<true, 2, false>, p)
+                       : cudaLaunchKernelEx(&cfg, k_sweep_inc64<false, 2, true>, p);
 }
 
 }  // namespace gpk
