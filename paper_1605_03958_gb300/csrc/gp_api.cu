@@ -1520,13 +1520,16 @@ int gp_observables(gp_solver* s, gp_obs* out) {
   if (const int rc_ = take_put(s)) return rc_;   // a pending overlapped write first
   wait_copies(s);
   const FieldParams f = field_params(s);
-  cudaError_t e = is_f64(s) ? gpk::launch_observables<double>(f, s->is_complex, s->stream)
-                            : gpk::launch_observables<float>(f, s->is_complex, s->stream);
-  if (e != cudaSuccess) return cuda_fail(s, e, "observables");
-  double o[10];
-  GP_CUDA(s, cudaMemcpyAsync(o, s->obs, sizeof o, cudaMemcpyDeviceToHost, s->stream));
-  const int rc = check_status(s);
-  if (rc != GP_OK) return rc;
+  double o[12];
+  for (bool two = gpk::observables_two(f);; two = false) {
+    const cudaError_t e = is_f64(s) ? gpk::launch_observables<double>(f, s->is_complex, two, s->stream)
+                                    : gpk::launch_observables<float>(f, s->is_complex, two, s->stream);
+    if (e != cudaSuccess) return cuda_fail(s, e, "observables");
+    GP_CUDA(s, cudaMemcpyAsync(o, s->obs, sizeof o, cudaMemcpyDeviceToHost, s->stream));
+    const int rc = check_status(s);
+    if (rc != GP_OK) return rc;
+    if (!two || gpk::observables_hold(o)) break;
+  }
   out->norm = o[0];
   out->mu = o[1];
   out->energy = o[2];
@@ -1546,8 +1549,8 @@ int gp_density2d(gp_solver* s, int plane, double* out) {
   wait_copies(s);
   const gp_params& p = s->prm;
   const FieldParams f = field_params(s);
-  cudaError_t e = is_f64(s) ? gpk::launch_density2d<double>(f, s->is_complex, plane, s->staging, s->stream)
-                            : gpk::launch_density2d<float>(f, s->is_complex, plane, s->staging, s->stream);
+  const cudaError_t e = is_f64(s) ? gpk::launch_density<double>(f, s->is_complex, plane, s->staging, s->stream)
+                                  : gpk::launch_density<float>(f, s->is_complex, plane, s->staging, s->stream);
   if (e != cudaSuccess) return cuda_fail(s, e, "density2d");
   const size_t n = plane == 0 ? (size_t)p.nx * p.ny : plane == 1 ? (size_t)p.nx * p.nz
                                                                  : (size_t)p.ny * p.nz;
@@ -1561,20 +1564,11 @@ int gp_density1d(gp_solver* s, int axis, double* out) {
   wait_copies(s);
   const gp_params& p = s->prm;
   const FieldParams f = field_params(s);
-  const int plane = axis == 2 ? 1 : 0;  // x, y from the xy plane; z from the xz plane
-  cudaError_t e = is_f64(s) ? gpk::launch_density2d<double>(f, s->is_complex, plane, s->staging, s->stream)
-                            : gpk::launch_density2d<float>(f, s->is_complex, plane, s->staging, s->stream);
-  if (e != cudaSuccess) return cuda_fail(s, e, "density2d");
-  double* red = s->staging + (size_t)p.nx * std::max(p.ny, p.nz);
-  if (axis == 0)
-    e = gpk::launch_cols_sum(s->staging, p.ny, p.nx, p.dy, red, s->stream);   // sum over y
-  else if (axis == 1)
-    e = gpk::launch_rows_sum(s->staging, p.ny, p.nx, p.dx, red, s->stream);   // sum over x
-  else
-    e = gpk::launch_rows_sum(s->staging, p.nz, p.nx, p.dx, red, s->stream);   // sum over x
+  const cudaError_t e = is_f64(s) ? gpk::launch_density<double>(f, s->is_complex, 3 + axis, s->staging, s->stream)
+                                  : gpk::launch_density<float>(f, s->is_complex, 3 + axis, s->staging, s->stream);
   if (e != cudaSuccess) return cuda_fail(s, e, "density1d");
   const size_t n = axis == 0 ? p.nx : axis == 1 ? p.ny : p.nz;
-  GP_CUDA(s, cudaMemcpyAsync(out, red, n * 8, cudaMemcpyDeviceToHost, s->stream));
+  GP_CUDA(s, cudaMemcpyAsync(out, s->staging, n * 8, cudaMemcpyDeviceToHost, s->stream));
   return check_status(s);
 }
 

@@ -698,12 +698,15 @@ int gp_pool_step(gp_pool* P, long nsteps) {
 int gp_pool_observables(gp_pool* P, int slot, gp_obs* out) {
   if (!slot_ok(P, slot) || !out) return P ? pfail(P, GP_ERR_ARG, "no such live slot or out is NULL") : GP_ERR_ARG;
   const FieldParams f = slot_field(P, slot);
-  cudaError_t e = gpk::launch_observables<float>(f, P->slots[slot].mode == 1, P->stream);
-  if (e != cudaSuccess) return pcuda(P, e, "observables");
-  double o[10];
-  PCUDA(P, cudaMemcpyAsync(o, P->d_obs, sizeof o, cudaMemcpyDeviceToHost, P->stream));
-  const int rc = check_status(P);
-  if (rc != GP_OK) return rc;
+  double o[12];
+  for (bool two = gpk::observables_two(f);; two = false) {
+    const cudaError_t e = gpk::launch_observables<float>(f, P->slots[slot].mode == 1, two, P->stream);
+    if (e != cudaSuccess) return pcuda(P, e, "observables");
+    PCUDA(P, cudaMemcpyAsync(o, P->d_obs, sizeof o, cudaMemcpyDeviceToHost, P->stream));
+    const int rc = check_status(P);
+    if (rc != GP_OK) return rc;
+    if (!two || gpk::observables_hold(o)) break;
+  }
   out->norm = o[0];
   out->mu = o[1];
   out->energy = o[2];

@@ -251,7 +251,16 @@ cudaError_t launch_inc64(int axis, const SweepParams& p, bool complex_field, cud
 // Resident warps per SM of the streaming y / z kernel (occupancy calculator).
 int stream_warps_per_sm(int axis, bool complex_field, int trunc);
 
-template <class R> cudaError_t launch_observables(const FieldParams& p, bool complex_field,
+// Observables into p.out[0..9] (gp_obs order).  With `two` (grids for which observables_two
+// holds) by two-part FP32 sums, p.out[10] receiving the field's largest |component| and
+// p.out[11] the pending factor: the result holds if observables_hold, else the call is
+// repeated without.
+bool observables_two(const FieldParams& p);
+inline bool observables_hold(const double* out) {
+  const double m = out[10], n = m * out[11];
+  return m >= 0x1p-16 && m <= 0x1p24 && n >= 0x1p-16 && n <= 0x1p24;
+}
+template <class R> cudaError_t launch_observables(const FieldParams& p, bool complex_field, bool two,
                                                   cudaStream_t st);
 // Standalone pointwise substep over the field (Strang splitting's half steps): trap
 // factors fx [pitch] and fyz [rows] of the half step, dtg = (dt / 2) g; the pending
@@ -277,12 +286,11 @@ template <class R> cudaError_t launch_import(const FieldParams& p, const double*
                                              bool complex_field, cudaStream_t st);
 template <class R> cudaError_t launch_export(const FieldParams& p, double* dst,
                                              bool complex_field, bool as_complex, cudaStream_t st);
-template <class R> cudaError_t launch_density2d(const FieldParams& p, bool complex_field,
-                                                int plane, double* out, cudaStream_t st);
-cudaError_t launch_rows_sum(const double* in, int rows, int cols, double w, double* out,
-                            cudaStream_t st);
-cudaError_t launch_cols_sum(const double* in, int rows, int cols, double w, double* out,
-                            cudaStream_t st);
+// |psi|^2 summed: which 0 over z (out[ny][nx]), 1 over y ([nz][nx]), 2 over x ([nz][ny]),
+// 3 over y and z ([nx]), 4 over x and z ([ny]), 5 over x and y ([nz]); out is followed by
+// room for the partial sums (in all at most the field's points in FP64 plus out).
+template <class R> cudaError_t launch_density(const FieldParams& p, bool complex_field, int which,
+                                              double* out, cudaStream_t st);
 
 // Message returned by gp_last_error(NULL) on this thread (gp_api.cu).
 void set_thread_error(const char* msg);

@@ -6,7 +6,10 @@
 // Every reduction runs on a fixed launch shape (kReduceBlocks x kReduceThreads),
 // sums in a fixed order (per thread, then a shuffle tree, then the blocks' partials
 // in index order by the last block to finish), and is therefore deterministic.
+#include <algorithm>
+
 #include "gp_device.cuh"
+#include "gp_split.cuh"
 
 namespace gpk {
 
@@ -148,6 +151,199 @@ __global__ void __launch_bounds__(kReduceThreads) k_observables(const FieldParam
     o[7] = sqrt(y2);
     o[8] = sqrt(z2);
     o[9] = sqrt(x2 + y2 + z2);
+  }
+}
+
+// ------------------------------------- observables in two-part FP32 sums
+
+// The same sums with the arithmetic on the FP32 pipe (gp_split.cuh: FP64 operations and
+// conversions run at 1/64 of FP32's rate here, and k_observables spends 32-45 of them per
+// point: 590 us for 240 x 200 x 160 complex64 points, where reading the field takes 9 us).
+// FP32 values are taken as they are, FP64 ones as two FP32 parts (48 bits, rounded to
+// nearest, so the terms' errors are independent and average out over the field); squares
+// and sums are two-part (2^-48 per addition), one FP64 conversion per thread and sum.  The
+// weights are exact: x^2 = (2i - nx + 1)^2 h^2 / 4 with the integer part in FP32, and the
+// potential energy follows from the three weighted sums.  The pending factor is applied
+// to the sums.  Fields whose largest value (times the factor) lies outside
+// [2^-16, 2^24], where sums of weighted fourth powers could leave FP32's range, and small grids (fewer than
+// 2^15 points, where k_observables takes no longer and there is less to average over) go
+// to k_observables; out[10] receives the largest |component| and out[11] the factor for the
+// host's check.
+// Measured (240 x 200 x 160, the whole call): complex64 736 -> 138 us, FP64 real 451 -> 112,
+// complex128 611 -> 170; the kernel (complex64, 110 us) is bound by its 216 instructions per
+// point, FP32 39 % of the pipe.  Error of the sums against quadruple precision at most a few
+// 1e-16 relative, as before (160 x 120 x 100 FP64: energy 1.3e-16, norm 2.6e-16).
+// A warp takes a row at a time, consecutive warps consecutive rows (y neighbours from L1),
+// the next 32 columns' loads in flight.
+constexpr int kObsTwoBlocks = 304;   // two resident blocks per SM
+
+template <class R, bool CPLX> struct PairLoad;   // columns (2c, 2c + 1), or (re, im) of column c
+template <bool CPLX> struct PairLoad<float, CPLX> {
+  using V = float2;
+  static __device__ __forceinline__ V load(const void* row, int c, int nc) {   // zero from nc on
+    return c < nc ? static_cast<const float2*>(row)[c] : f2(0.f);
+  }
+  static __device__ __forceinline__ Two two(V v, int c, int nx) {
+    if (!CPLX && 2 * c + 1 >= nx) v.y = 0.f;
+    return two_scalar(v, f2(0.f));
+  }
+};
+template <bool CPLX> struct PairLoad<double, CPLX> {
+  using V = double2;
+  static __device__ __forceinline__ V load(const void* row, int c, int nc) {
+    return c < nc ? static_cast<const double2*>(row)[c] : make_double2(0.0, 0.0);
+  }
+  static __device__ __forceinline__ Two two(V v, int c, int nx) {
+    if (!CPLX && 2 * c + 1 >= nx) v.y = 0.0;
+    int tmax = 0;
+    const Two t = split2(v.x, v.y, &tmax);
+    // out of range: an infinity, for the host's check
+    const float s = tmax >= kSplitTooBig ? __int_as_float(0x7f800000) : 0x1p-56f;
+    return two_scalar(mul2(t.h, f2(s)), mul2(t.l, f2(s)));
+  }
+};
+
+template <class R, bool CPLX>
+__global__ void __launch_bounds__(kReduceThreads, 2) k_observables_two(const FieldParams p) {
+  const int nx = p.nx, ny = p.ny, nz = p.nz;
+  const int nc = CPLX ? nx : (nx + 1) / 2;   // column pairs
+  const size_t rowb = (size_t)p.pitch * sizeof(R) * (CPLX ? 2 : 1);
+  const unsigned char* field = static_cast<const unsigned char*>(p.psi);
+  const int lane = threadIdx.x & 31;
+  const int nrows = ny * nz;
+  using L = PairLoad<R, CPLX>;
+  constexpr bool LOW = sizeof(R) == 8;   // values have low parts
+  // v^2 without the square of the low part, which (never negative) would always round away:
+  // those are summed by themselves in `low`; renormalised, so that the sums' low parts stay
+  // small
+  auto square = [](const Two& v, float2* low) {
+    Two q;
+    q.h = mul2(v.h, v.h);
+    q.l = fma2(add2(v.h, v.h), v.l, fma2(v.h, v.h, mul2(q.h, f2(-1.f))));
+    *low = fma2(v.l, v.l, *low);
+    return two_scalar(add2(q.h, q.l), sub2(q.l, sub2(add2(q.h, q.l), q.h)));
+  };
+  auto edge = [&](const Two& a, const Two& b, float2* low) {   // |a - b|^2
+    Two d;
+    float2 e;
+    const Two n = two_neg(b);
+    two_sum(a.h, n.h, &d.h, &e);
+    d.l = LOW ? add2(add2(a.l, n.l), e) : e;
+    return square(d, low);
+  };
+  float2 lSX = f2(0.f), lS4 = f2(0.f), lX = f2(0.f), lY = f2(0.f), lZ = f2(0.f);
+  Two S = two_zero(), SX = two_zero(), SY = two_zero(), SZ = two_zero(), S4 = two_zero(), KX = two_zero(),
+      KY = two_zero(), KZ = two_zero();
+  float vmax = 0.f;
+  const int step = gridDim.x * (kReduceThreads / 32);
+  for (int r = blockIdx.x * (kReduceThreads / 32) + (threadIdx.x >> 5); r < nrows; r += step) {
+    const int k = r / ny, j = r - k * ny;
+    const unsigned char* row = field + (size_t)r * rowb;
+    Two SR = two_zero();
+    float2 lSR = f2(0.f);
+    auto fetch = [&](int c, typename L::V (&b)[4]) {   // a point and its three neighbours
+      b[0] = L::load(row, c, nc);
+      b[1] = L::load(row, c + 1, nc);
+      b[2] = L::load(row + rowb, c, j + 1 < ny ? nc : 0);
+      b[3] = L::load(row + rowb * ny, c, k + 1 < nz ? nc : 0);
+    };
+    typename L::V cur[4], ahead[4];
+    fetch(lane, cur);
+    for (int c = lane; c < nc; c += 32) {
+      fetch(c + 32, ahead);
+      const Two v = L::two(cur[0], c, nx), nxt = L::two(cur[1], c + 1, nx), wy = L::two(cur[2], c, nx),
+                wz = L::two(cur[3], c, nx);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) cur[q] = ahead[q];
+      const Two wx = CPLX ? nxt : two_scalar(f2(v.h.y, nxt.h.x), f2(v.l.y, nxt.l.x));
+      vmax = fmaxf(vmax, fmaxf(fabsf(v.h.x), fabsf(v.h.y)));
+      float2 ll = f2(0.f);
+      const Two q = square(v, &ll);
+      SR = two_add(SR, q);
+      lSR = add2(lSR, ll);
+      // (2i - nx + 1)^2 below 2^22: exact in FP32
+      const float w0 = (float)(2 * (CPLX ? c : 2 * c) - nx + 1), w1 = CPLX ? w0 : w0 + 2.f;
+      const float2 wc = f2(w0 * w0, w1 * w1);
+      SX = two_add(SX, two_mul(two_scalar(wc, f2(0.f)), q));
+      const Two d = CPLX ? two_add(q, two_swap(q)) : q;
+      S4 = two_add(S4, square(d, &lS4));
+      if (LOW) {   // the squares of the values' low parts in the weighted and fourth-power sums
+        lSX = fma2(wc, ll, lSX);
+        lS4 = fma2(add2(d.h, d.h), CPLX ? add2(ll, f2(ll.y, ll.x)) : ll, lS4);
+      }
+      KX = two_add(KX, edge(wx, v, &lX));
+      KY = two_add(KY, edge(wy, v, &lY));
+      KZ = two_add(KZ, edge(wz, v, &lZ));
+      if (c == 0) {   // the ghost edge at i = 0
+        const float2 m = f2(1.f, CPLX ? 1.f : 0.f);
+        KX = two_add(KX, two_scalar(mul2(q.h, m), mul2(q.l, m)));
+      }
+      if (j == 0) KY = two_add(KY, q);
+      if (k == 0) KZ = two_add(KZ, q);
+    }
+    if (LOW) SR = two_add(SR, two_scalar(lSR, f2(0.f)));
+    S = two_add(S, SR);
+    const float wj = (float)(2 * j - ny + 1), wk = (float)(2 * k - nz + 1);
+    SY = two_add(SY, two_mul(two_scalar(f2(wj * wj), f2(0.f)), SR));
+    SZ = two_add(SZ, two_mul(two_scalar(f2(wk * wk), f2(0.f)), SR));
+  }
+  auto total = [](const Two& t, bool both) {
+    const Two n = two_norm(t);
+    if (!(fabsf(n.h.x) + fabsf(n.h.y) <= 1e30f)) return (double)__int_as_float(0x7fc00000);   // NaN among the values
+    const double a = to_double(n.h.x, n.l.x, kSplitShift);
+    return both ? a + to_double(n.h.y, n.l.y, kSplitShift) : a;
+  };
+  auto with = [](const Two& t, float2 low) { return two_add(t, two_scalar(low, f2(0.f))); };
+  SX = with(SX, lSX);
+  S4 = with(S4, lS4);
+  KX = with(KX, lX);
+  KY = with(KY, lY);
+  KZ = with(KZ, lZ);
+  double acc[8] = {total(S, true),        total(SX, true), total(SY, true), total(SZ, true),
+                   total(S4, !CPLX), total(KX, true), total(KY, true), total(KZ, true)};
+  const unsigned int wmax = __reduce_max_sync(0xffffffffu, __float_as_uint(vmax));
+  __shared__ unsigned int bmax;
+  if (threadIdx.x == 0) bmax = 0u;
+  __syncthreads();
+  if (lane == 0) atomicMax(&bmax, wmax);
+  __syncthreads();
+  double* maxima = p.partials + (size_t)gridDim.x * 8;
+  if (threadIdx.x == 0) maxima[blockIdx.x] = (double)__uint_as_float(bmax);
+  __shared__ double tot[8];
+  if (!block_reduce_last<8>(acc, p.partials, p.counter, tot)) return;
+  unsigned int m = 0u;
+  for (unsigned int b = threadIdx.x; b < gridDim.x; b += blockDim.x)
+    m = max(m, __float_as_uint((float)__ldcg(maxima + b)));
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) atomicMax(&bmax, m);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const double s = *p.scale, s2 = s * s, dV = p.hx * p.hy * p.hz;
+    const double* Vx = p.tab;
+    const double* X2 = Vx + nx + ny + nz;
+    const double sum = tot[0] * s2, norm = sum * dV;
+    const double sx = tot[1] * s2 * (0.25 * p.hx * p.hx), sy = tot[2] * s2 * (0.25 * p.hy * p.hy);
+    const double sz = nz == 1 ? 0.0 : tot[3] * s2 * (0.25 * p.hz * p.hz);
+    // V_a(x) = (w_a^2 / 2) x^2: the tables' ratio at the first point (nonzero there)
+    const double epot = (sx * (Vx[0] / X2[0]) + sy * (Vx[nx] / X2[nx]) +
+                         (nz == 1 ? 0.0 : sz * (Vx[nx + ny] / X2[nx + ny]))) * dV;
+    const double eint = 0.5 * p.g * (tot[4] * s2 * s2) * dV;
+    const double ekin = 0.5 * dV * s2 * (tot[5] / (p.hx * p.hx) + tot[6] / (p.hy * p.hy) +
+                                         (nz == 1 ? 0.0 : tot[7] / (p.hz * p.hz)));
+    const double x2 = sx * dV / norm, y2 = sy * dV / norm, z2 = sz * dV / norm;
+    double* o = p.out;
+    o[0] = norm;
+    o[1] = ekin + epot + 2.0 * eint;
+    o[2] = ekin + epot + eint;
+    o[3] = ekin;
+    o[4] = epot;
+    o[5] = eint;
+    o[6] = sqrt(x2);
+    o[7] = sqrt(y2);
+    o[8] = sqrt(z2);
+    o[9] = sqrt(x2 + y2 + z2);
+    o[10] = (double)__uint_as_float(bmax);
+    o[11] = s;
   }
 }
 
@@ -342,42 +538,197 @@ __global__ void k_export(const FieldParams p, double* __restrict__ dst, int as_c
 
 // ------------------------------------------------------- integrated densities
 
-// plane 0: out[j*nx+i] = dz sum_k |psi|^2 ; plane 1: out[k*nx+i] = dy sum_j |psi|^2
+// |psi|^2 summed along one direction, kDensSum terms per thread: chunk ch of the nsum
+// rows `step` elements apart, for every column and each of the rows_out starting rows
+// `out_step` apart; part[(ch rows_out + o) nx + i].  One 16-byte vector per thread and
+// row.  FP64 work is what the sums must not wait for (see k_observables_two): FP32 values
+// are squared and added in two FP32 parts, eight terms at a time (their errors, about 2^-50
+// of the eight, average out over a chunk's and the chunks' FP64 additions), then added
+// in FP64; FP64 values cost one or two FP64 operations each.  The factor is applied by
+// the final sum.  Measured (240 x 200 x 160 complex64, the whole call): 202-239 -> 45-55 us
+// per density, of which the kernels take 16-20 us.
+constexpr int kDensSum = 32;
 template <class R, bool CPLX>
-__global__ void k_density_sum_strided(const FieldParams p, int plane, double* __restrict__ out) {
-  const int nx = p.nx, ny = p.ny, nz = p.nz;
-  const size_t P = (size_t)p.pitch;
-  const double s = *p.scale;
-  const int rows = plane == 0 ? ny : nz;          // output rows
-  const int nsum = plane == 0 ? nz : ny;          // summed extent
-  const size_t step = plane == 0 ? P * ny : P;    // stride of the summed axis
-  const double w = plane == 0 ? p.hz : p.hy;
-  const long long total = (long long)rows * nx;
-  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < total;
-       q += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(q % nx), o = (int)(q / nx);
-    const size_t base = plane == 0 ? (size_t)o * P + i : (size_t)o * P * ny + i;
-    double acc = 0.0;
-    for (int t = 0; t < nsum; ++t) acc += dabs2(Load<R, CPLX>::at(p.psi, base + t * step, s));
-    out[q] = acc * w;
+__global__ void __launch_bounds__(128) k_density_partial(const FieldParams p, int rows_out, size_t out_step,
+                                                         int nsum, size_t step, double* __restrict__ part) {
+  constexpr int W = 16 / (int)sizeof(R) / (CPLX ? 2 : 1);   // columns per vector
+  const int nx = p.nx, nvec = (nx + W - 1) / W;
+  const unsigned int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned int xv = t % (unsigned int)nvec, rest = t / (unsigned int)nvec;
+  const int o = (int)(rest % (unsigned int)rows_out), ch = (int)(rest / (unsigned int)rows_out);
+  const int r0 = ch * kDensSum, r1 = min(nsum, r0 + kDensSum);
+  if (r0 >= nsum) return;
+  constexpr int EB = (int)sizeof(R) * (CPLX ? 2 : 1);
+  const float4* src = reinterpret_cast<const float4*>(static_cast<const unsigned char*>(p.psi) +
+                                                      ((size_t)o * out_step + (size_t)xv * W) * EB);
+  const size_t sv = step * EB / 16;
+  double acc[W];
+#pragma unroll
+  for (int e = 0; e < W; ++e) acc[e] = 0.0;
+  for (int r = r0; r < r1; r += 8) {
+    float4 v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = r + q < r1 ? src[(size_t)(r + q) * sv] : make_float4(0.f, 0.f, 0.f, 0.f);
+    if constexpr (sizeof(R) == 8) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const double2 d = *reinterpret_cast<const double2*>(&v[q]);
+        if (CPLX) {
+          acc[0] = fma(d.x, d.x, fma(d.y, d.y, acc[0]));
+        } else {
+          acc[0] = fma(d.x, d.x, acc[0]);
+          acc[W - 1] = fma(d.y, d.y, acc[W - 1]);
+        }
+      }
+    } else {
+      // values are scaled by a power of two that takes the largest of the eight vectors to
+      // about 1, which keeps the squares in FP32's range
+      float m = 0.f;
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        m = fmaxf(fmaxf(fmaxf(m, fabsf(v[q].x)), fmaxf(fabsf(v[q].y), fabsf(v[q].z))), fabsf(v[q].w));
+      const int ex = min(max((int)(__float_as_uint(m) >> 23), 30), 223);
+      const float2 sc = f2(__uint_as_float((unsigned int)(254 - ex) << 23));
+      Two s0 = two_zero(), s1 = two_zero();
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const float2 a = mul2(f2(v[q].x, v[q].y), sc), b = mul2(f2(v[q].z, v[q].w), sc);
+        Two qa, qb;
+        qa.h = mul2(a, a);
+        qa.l = fma2(a, a, mul2(qa.h, f2(-1.f)));
+        qb.h = mul2(b, b);
+        qb.l = fma2(b, b, mul2(qb.h, f2(-1.f)));
+        s0 = two_add(s0, qa);
+        s1 = two_add(s1, qb);
+      }
+      if (CPLX) {
+        s0 = two_add(s0, two_swap(s0));
+        s1 = two_add(s1, two_swap(s1));
+      }
+      s0 = two_norm(s0);
+      s1 = two_norm(s1);
+      const int k = kSplitShift + 2 * (ex - 127);
+      if (fabsf(s0.h.x) + fabsf(s0.h.y) + fabsf(s1.h.x) + fabsf(s1.h.y) <= 1e30f) {
+        acc[0] += to_double(s0.h.x, s0.l.x, k);
+        if (CPLX) {
+          acc[1 % W] += to_double(s1.h.x, s1.l.x, k);
+        } else {
+          acc[1 % W] += to_double(s0.h.y, s0.l.y, k);
+          acc[2 % W] += to_double(s1.h.x, s1.l.x, k);
+          acc[3 % W] += to_double(s1.h.y, s1.l.y, k);
+        }
+      } else {   // infinities or NaN among the values
+        for (int q = 0; q < 8; ++q) {
+          const float e[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+          for (int i = 0; i < 4; ++i) acc[CPLX ? i / 2 % W : i % W] += (double)e[i] * (double)e[i];
+        }
+      }
+    }
+  }
+  double* dst = part + ((size_t)ch * rows_out + o) * nx + (size_t)xv * W;
+#pragma unroll
+  for (int e = 0; e < W; ++e)
+    if ((int)xv * W + e < nx) dst[e] = acc[e];
+}
+
+// out[q] = w scale^2 sum over ch of part[ch total + q], q < total: blockDim.x outputs per
+// block, each of its rows of threads on every blockDim.y-th chunk, then added in order.
+// (Few outputs of many chunks: 8 x 64 threads, so that the FP64 additions spread over
+// more SMs; 240 sums of 1000 chunks took 22 us on 8 blocks of 32 outputs.)
+__global__ void __launch_bounds__(512) k_density_combine(const double* __restrict__ part, int nch,
+                                                         long long total, double w, const double* scale,
+                                                         double* __restrict__ out) {
+  __shared__ double sm[64 * 9];
+  const int bx = blockDim.x, by = blockDim.y;
+  const long long q = (long long)blockIdx.x * bx + threadIdx.x;
+  double acc = 0.0;
+  if (q < total)
+#pragma unroll 4
+    for (int c = threadIdx.y; c < nch; c += by) acc += part[(size_t)c * total + q];
+  sm[threadIdx.y * (bx + 1) + threadIdx.x] = acc;
+  __syncthreads();
+  if (threadIdx.y == 0 && q < total) {
+    double v = sm[threadIdx.x];
+    for (int t = 1; t < by; ++t) v += sm[t * (bx + 1) + threadIdx.x];
+    const double s = scale ? *scale : 1.0;
+    out[q] = v * (w * s * s);
   }
 }
 
-// plane 2: out[k*ny+j] = dx sum_i |psi|^2, one warp per (j, k) row
+// out[r] = w sum_i |psi|^2 of row r = k ny + j, eight rows per warp: the lanes' sums of the
+// eight are added by a butterfly that halves the rows a lane carries at every exchange
+// (nine FP64 additions for eight rows; forty with a tree per row made FP64 the bound).
 template <class R, bool CPLX>
-__global__ void k_density_sum_rows(const FieldParams p, double* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_density_sum_rows(const FieldParams p, double w, double* __restrict__ out) {
   const int lane = threadIdx.x & 31;
-  const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-  const long long nrows = (long long)p.ny * p.nz;
+  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nrows = p.ny * p.nz;
+  const int r0 = 8 * warp;
+  if (r0 >= nrows) return;
   const double s = *p.scale;
-  for (long long r = warp; r < nrows; r += nwarps) {
+  const int nc = CPLX ? p.nx : (p.nx + 1) / 2;   // column pairs
+  double sum[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
     double acc = 0.0;
-    for (int i = lane; i < p.nx; i += 32)
-      acc += dabs2(Load<R, CPLX>::at(p.psi, (size_t)r * p.pitch + i, s));
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if (lane == 0) out[r] = acc * p.hx;
+    const R* base = static_cast<const R*>(p.psi) + (size_t)(r0 + t) * p.pitch * (CPLX ? 2 : 1);
+    const int n = r0 + t < nrows ? nc : 0;
+    if constexpr (sizeof(R) == 8) {
+      const double2* row = reinterpret_cast<const double2*>(base);
+      for (int c = lane; c < n; c += 32) {
+        double2 v = row[c];
+        if (!CPLX && 2 * c + 1 >= p.nx) v.y = 0.0;
+        acc = fma(v.x, v.x, fma(v.y, v.y, acc));
+      }
+    } else {
+      const float2* row = reinterpret_cast<const float2*>(base);
+      for (int c0 = lane; c0 < n; c0 += 32 * 8) {   // eight pairs in two parts, as k_density_partial
+        float2 v[8];
+        float m = 0.f;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int c = c0 + 32 * q;
+          v[q] = c < n ? row[c] : f2(0.f);
+          if (!CPLX && 2 * c + 1 >= p.nx) v[q].y = 0.f;
+          m = fmaxf(m, fmaxf(fabsf(v[q].x), fabsf(v[q].y)));
+        }
+        const int ex = min(max((int)(__float_as_uint(m) >> 23), 30), 223);
+        const float2 sc = f2(__uint_as_float((unsigned int)(254 - ex) << 23));
+        Two s0 = two_zero();
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const float2 a = mul2(v[q], sc);
+          Two qa;
+          qa.h = mul2(a, a);
+          qa.l = fma2(a, a, mul2(qa.h, f2(-1.f)));
+          s0 = two_add(s0, qa);
+        }
+        s0 = two_norm(two_add(s0, two_swap(s0)));
+        if (fabsf(s0.h.x) <= 1e30f) {
+          acc += to_double(s0.h.x, s0.l.x, kSplitShift + 2 * (ex - 127));
+        } else {   // infinities or NaN among the values
+          for (int q = 0; q < 8; ++q)
+            acc = fma((double)v[q].x, (double)v[q].x, fma((double)v[q].y, (double)v[q].y, acc));
+        }
+      }
+    }
+    sum[t] = acc;
   }
+  // lane bits 4, 3, 2 choose the row that a lane ends up with, bits 1 and 0 the quarter
+#pragma unroll
+  for (int half = 4, bit = 16; half >= 1; half >>= 1, bit >>= 1) {
+    const bool up = (lane & bit) != 0;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      if (t >= half) break;
+      const double keep = up ? sum[t + half] : sum[t], give = up ? sum[t] : sum[t + half];
+      sum[t] = keep + __shfl_xor_sync(0xffffffffu, give, bit);
+    }
+  }
+  double v = sum[0];
+  v += __shfl_xor_sync(0xffffffffu, v, 2);
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  const int r = r0 + (lane >> 2);
+  if ((lane & 3) == 0 && r < nrows) out[r] = v * (w * s * s);
 }
 
 // out[r] = w * sum_c in[r*cols + c], one warp per row
@@ -392,16 +743,6 @@ __global__ void k_rows_sum(const double* __restrict__ in, int rows, int cols, do
   if (lane == 0) out[warp] = acc * w;
 }
 
-// out[c] = w * sum_r in[r*cols + c], one thread per column
-__global__ void k_cols_sum(const double* __restrict__ in, int rows, int cols, double w,
-                           double* __restrict__ out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  double acc = 0.0;
-  for (int r = 0; r < rows; ++r) acc += in[(size_t)r * cols + c];
-  out[c] = acc * w;
-}
-
 // ---------------------------------------------------------------- launchers
 
 static unsigned int grid_for_rows(const FieldParams& p) {
@@ -409,8 +750,19 @@ static unsigned int grid_for_rows(const FieldParams& p) {
   return (unsigned int)(nrows < 4096 ? nrows : 4096);
 }
 
+bool observables_two(const FieldParams& p) {
+  return (long long)p.nx * p.ny * p.nz >= (1LL << 15);
+}
+
 template <class R>
-cudaError_t launch_observables(const FieldParams& p, bool complex_field, cudaStream_t st) {
+cudaError_t launch_observables(const FieldParams& p, bool complex_field, bool two, cudaStream_t st) {
+  if (two) {
+    if (complex_field)
+      k_observables_two<R, true><<<kObsTwoBlocks, kReduceThreads, 0, st>>>(p);
+    else
+      k_observables_two<R, false><<<kObsTwoBlocks, kReduceThreads, 0, st>>>(p);
+    return cudaGetLastError();
+  }
   if (complex_field)
     k_observables<R, true><<<kReduceBlocks, kReduceThreads, 0, st>>>(p);
   else
@@ -492,39 +844,57 @@ cudaError_t launch_export(const FieldParams& p, double* dst, bool complex_field,
   return cudaGetLastError();
 }
 
+static void launch_combine(const double* part, int nch, long long total, double w, const double* scale,
+                           double* out, cudaStream_t st) {
+  const dim3 block = nch <= 16 ? dim3(32, 8) : dim3(8, 64);
+  k_density_combine<<<(unsigned int)((total + block.x - 1) / block.x), block, 0, st>>>(part, nch, total, w, scale, out);
+}
+
+// |psi|^2 over the lines of a direction into out (see launch_density): the partial sums go
+// behind it
 template <class R>
-cudaError_t launch_density2d(const FieldParams& p, bool complex_field, int plane, double* out,
-                             cudaStream_t st) {
-  if (plane == 2) {
-    if (complex_field)
-      k_density_sum_rows<R, true><<<1024, 256, 0, st>>>(p, out);
-    else
-      k_density_sum_rows<R, false><<<1024, 256, 0, st>>>(p, out);
-  } else {
-    if (complex_field)
-      k_density_sum_strided<R, true><<<1024, 256, 0, st>>>(p, plane, out);
-    else
-      k_density_sum_strided<R, false><<<1024, 256, 0, st>>>(p, plane, out);
+static cudaError_t density_lines(const FieldParams& p, bool complex_field, int rows_out, size_t out_step,
+                                 int nsum, size_t step, double w, double* out, cudaStream_t st) {
+  const int W = 16 / (int)sizeof(R) / (complex_field ? 2 : 1);
+  const int nvec = (p.nx + W - 1) / W, nch = (nsum + kDensSum - 1) / kDensSum;
+  const long long total = (long long)rows_out * p.nx;
+  double* part = out + total;
+  const unsigned int blocks = (unsigned int)(((long long)nvec * rows_out * nch + 127) / 128);
+  if (complex_field)
+    k_density_partial<R, true><<<blocks, 128, 0, st>>>(p, rows_out, out_step, nsum, step, part);
+  else
+    k_density_partial<R, false><<<blocks, 128, 0, st>>>(p, rows_out, out_step, nsum, step, part);
+  launch_combine(part, nch, total, w, p.scale, out, st);
+  return cudaGetLastError();
+}
+
+template <class R>
+cudaError_t launch_density(const FieldParams& p, bool complex_field, int which, double* out, cudaStream_t st) {
+  const size_t P = (size_t)p.pitch, plane = P * (size_t)p.ny;
+  switch (which) {
+    case 0: return density_lines<R>(p, complex_field, p.ny, P, p.nz, plane, p.hz, out, st);
+    case 1: return density_lines<R>(p, complex_field, p.nz, plane, p.ny, P, p.hy, out, st);
+    case 3: return density_lines<R>(p, complex_field, 1, 0, p.ny * p.nz, P, p.hy * p.hz, out, st);
+    default: break;
+  }
+  const double w = which == 2 ? p.hx : which == 4 ? p.hx * p.hz : p.hx * p.hy;
+  const long long rows = (long long)p.ny * p.nz;
+  double* sums = which == 2 ? out : out + std::max(p.ny, p.nz);   // the rows' sums
+  const unsigned int blocks = (unsigned int)((rows + 63) / 64);   // eight warps of eight rows
+  if (complex_field)
+    k_density_sum_rows<R, true><<<blocks, 256, 0, st>>>(p, w, sums);
+  else
+    k_density_sum_rows<R, false><<<blocks, 256, 0, st>>>(p, w, sums);
+  if (which == 4) {   // over z: column j of [nz][ny]
+    launch_combine(sums, p.nz, p.ny, 1.0, nullptr, out, st);
+  } else if (which == 5) {   // over y: row k of [nz][ny]
+    k_rows_sum<<<(unsigned int)((p.nz + 7) / 8), 256, 0, st>>>(sums, p.nz, p.ny, 1.0, out);
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_rows_sum(const double* in, int rows, int cols, double w, double* out,
-                            cudaStream_t st) {
-  const int threads = 256, warps_per_block = threads / 32;
-  k_rows_sum<<<(rows + warps_per_block - 1) / warps_per_block, threads, 0, st>>>(in, rows, cols,
-                                                                                  w, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_cols_sum(const double* in, int rows, int cols, double w, double* out,
-                            cudaStream_t st) {
-  k_cols_sum<<<(cols + 255) / 256, 256, 0, st>>>(in, rows, cols, w, out);
-  return cudaGetLastError();
-}
-
 #define GP_INSTANTIATE(R)                                                                      \
-  template cudaError_t launch_observables<R>(const FieldParams&, bool, cudaStream_t);         \
+  template cudaError_t launch_observables<R>(const FieldParams&, bool, bool, cudaStream_t);   \
   template cudaError_t launch_norm_to_scale<R>(const FieldParams&, cudaStream_t);             \
   template cudaError_t launch_half_pointwise<R>(const FieldParams&, bool, const void*,       \
                                                 const void*, double, bool, bool, cudaStream_t); \
@@ -532,7 +902,7 @@ cudaError_t launch_cols_sum(const double* in, int rows, int cols, double w, doub
                                                cudaStream_t);                                  \
   template cudaError_t launch_import<R>(const FieldParams&, const double*, bool, cudaStream_t); \
   template cudaError_t launch_export<R>(const FieldParams&, double*, bool, bool, cudaStream_t); \
-  template cudaError_t launch_density2d<R>(const FieldParams&, bool, int, double*, cudaStream_t);
+  template cudaError_t launch_density<R>(const FieldParams&, bool, int, double*, cudaStream_t);
 GP_INSTANTIATE(double)
 GP_INSTANTIATE(float)
 #undef GP_INSTANTIATE
