@@ -385,13 +385,16 @@ int cuda_fail(gp_solver* s, cudaError_t e, const char* where) {
     if (e_ != cudaSuccess) return cuda_fail((s), e_, #call); \
   } while (0)
 
-// The factor of a solver whose z sweep defers its norm: sum the partials into it when
+// The sweep that ends a step: z, or y in 2D.
+int last_axis(const gp_solver* s) { return s->prm.nz == 1 ? 1 : 2; }
+
+// The factor of a solver whose last sweep defers its norm: sum the partials into it when
 // they are newer than it (one small kernel on the solver's stream; nothing otherwise).
 void resolve_scale(gp_solver* s) {
   if (!s->defer_norm) return;
   const cudaError_t e =
       gpk::launch_resolve_scale(s->scale, s->scale_state, s->partials,
-                                (int)s->fast_grid[0][2], s->prm.dx * s->prm.dy * s->prm.dz,
+                                (int)s->fast_grid[0][last_axis(s)], s->sp[0][0].dV,
                                 s->status, s->stream);
   if (e != cudaSuccess) cuda_fail(s, e, "resolve scale");
 }
@@ -490,7 +493,7 @@ void fill_sweep_params(gp_solver* s) {
       q.scale_out = s->scale;
       q.status = s->status;
       q.wait_ns = gpk::kWaitLimitNs;
-      q.dV = p.dx * p.dy * p.dz;
+      q.dV = p.dx * p.dy * (p.nz == 1 ? 1.0 : p.dz);
       q.ntiles = s->L.ntiles_z[m];
       if (s->line64 && (a < 2 || p.nz > 1)) {
         // the increment form where the line qualifies (one norm partial per block)
@@ -499,8 +502,9 @@ void fill_sweep_params(gp_solver* s) {
         q.inc_amax = reinterpret_cast<int*>(s->step_ctr) + 1;
         if (!gpk::inc64_setup(a, &q, m == 0 ? std::complex<double>(beta, 0.0)
                                              : std::complex<double>(0.0, beta), m == 1) ||
-            (a == 2 && gpk::inc64_blocks(a, q, m == 1) > (long long)s->L.npartials))
+            (a > 0 && gpk::inc64_blocks(a, q, m == 1) > (long long)s->L.npartials))
           q.inc_x = 0;
+        q.plane_norm = q.inc_x && p.nz == 1 && a == 1 && m == 0 ? 1 : 0;
       }
       q.trunc = s->trunc[m][a];
       if (q.trunc) {
@@ -572,7 +576,7 @@ void fill_sweep_params(gp_solver* s) {
         // rows measured no faster that way)
         int rbps = 0;
         if (q.band_w && m == 0 && gpk::x_reg_fits(p.nx, q.band_w) && x_reg_enabled() &&
-            gpk::x_reg_prepare(q.band_w, m == 1, &rbps) == cudaSuccess && rbps > 0) {
+            gpk::x_reg_prepare(q.band_w, p.nz == 1, &rbps) == cudaSuccess && rbps > 0) {
           const long long rows = (long long)p.ny * p.nz;
           const long long warps = std::min((long long)s->nsm * rbps * gpk::kXRegWarps, rows);
           q.band_rows = (int)(rows / warps);
@@ -598,7 +602,8 @@ void fill_sweep_params(gp_solver* s) {
         const long long cols = (long long)((p.nx + ept - 1) / ept) * (a == 1 ? p.nz : p.ny);
         q.band_cp = band_prefetch() ? 1 : 0;
         // (sets the kernel's shared-memory limit, above 48 KB at W = 8)
-        gpk::band_line_blocks_per_sm(a, m == 1, q.band_w, q.band_cp != 0);
+        q.plane_norm = p.nz == 1 && a == 1 && m == 0 ? 1 : 0;
+        gpk::band_line_blocks_per_sm(a, m == 1, q.plane_norm != 0, q.band_w, q.band_cp != 0);
         const int forced = band_seg_turns();
         int best_seg = std::min((forced > 0 ? forced : (10 + P - 1) / P) * P, std::max(n[a], P));
         // one FP64 norm partial per block must fit the partials area
@@ -611,17 +616,24 @@ void fill_sweep_params(gp_solver* s) {
         s->fast_grid[m][a] = (int)blocks;
       }
     }
-  // FP32 real field, banded x and z sweeps: the z sweep only stores its norm partials
-  // and the next x sweep sums them (every block, in the same order) into the factor it
-  // applies, instead of the last z block summing them at the end of the z sweep; other
-  // readers of the factor resolve it first (resolve_scale)
-  s->defer_norm = s->L.rbytes == 4 && p.nz > 1 && s->band_w[0][0] && s->band_w[0][2] &&
-                  norm_defer_enabled();
+  // 2D, banded x and y sweeps: x goes from the field to the staging area and y back, so
+  // that a step ends in the field without a copy
+  for (int m = 0; m < 2 && p.nz == 1; ++m)
+    if (s->band_w[m][0] && s->band_w[m][1]) {
+      s->sp[m][0].out = s->sp[m][1].psi = s->staging;
+      s->sp[m][1].out = s->field;
+    }
+  // FP32 real field, banded x sweep and banded last sweep (z; 2D: y): the last sweep only
+  // stores its norm partials and the next x sweep sums them (every block, in the same
+  // order) into the factor it applies, instead of the last block summing them at the end;
+  // other readers of the factor resolve it first (resolve_scale)
+  const int la = last_axis(s);
+  s->defer_norm = s->L.rbytes == 4 && s->band_w[0][0] && s->band_w[0][la] && norm_defer_enabled();
   for (int a = 0; a < 3; ++a) {
     SweepParams& q = s->sp[0][a];
-    q.norm_defer = s->defer_norm && a != 1 ? 1 : 0;
-    q.norm_blocks = s->fast_grid[0][2];
-    q.norm_copies = std::max(1, std::min(8, (int)(s->L.npartials / std::max(1, s->fast_grid[0][2]))));
+    q.norm_defer = s->defer_norm && (a == 0 || a == la) ? 1 : 0;
+    q.norm_blocks = s->fast_grid[0][la];
+    q.norm_copies = std::max(1, std::min(8, (int)(s->L.npartials / std::max(1, s->fast_grid[0][la]))));
     q.scale_state = s->scale_state;
   }
 }
@@ -940,7 +952,7 @@ template <class R> int run_sweep(gp_solver* s, int axis) {
   }
   cudaError_t e;
   if (axis == 0 && q.band_w && q.band_reg)
-    e = gpk::launch_sweep_x_reg(q, m == 1, s->fast_grid[m][0], s->stream);
+    e = gpk::launch_sweep_x_reg(q, s->fast_grid[m][0], s->stream);
   else if (axis == 0 && q.band_w)
     e = gpk::launch_sweep_x_band(q, m == 1, s->fast_grid[m][0], s->stream);
   else if (q.band_w)
@@ -972,14 +984,15 @@ template <class R> int lie_step_direct(gp_solver* s) {
   {
     for (int a = 0; a < 3; ++a) {
       if (a == 2 && two_d) {
-        // 2D: no z sweep.  A fast y sweep wrote the staging area: copy it back; then
-        // imaginary time renormalises with a norm pass over the plane
+        // 2D: no z sweep.  A fast y sweep that wrote the staging area: copy it back; then,
+        // unless the y sweep summed it, imaginary time renormalises with a norm pass over
+        // the plane
         const int m = s->is_complex ? 1 : 0;
-        if (s->sp[m][1].trunc || s->sp[m][1].band_w)
+        if ((s->sp[m][1].trunc || s->sp[m][1].band_w) && s->sp[m][1].out != s->field)
           GP_CUDA(s, cudaMemcpyAsync(s->field, s->staging,
                                      (size_t)s->L.pitch[m] * s->L.rbytes * (m + 1) * s->prm.ny,
                                      cudaMemcpyDeviceToDevice, s->stream));
-        if (!s->is_complex) {
+        if (!s->is_complex && !s->sp[0][1].plane_norm) {
           FieldParams f = field_params(s);
           f.out = s->scale;
           const cudaError_t e = gpk::launch_norm_to_scale<R>(f, s->stream);

@@ -66,7 +66,7 @@ constexpr int kObsAcc = 9;
 //   A_j = m_j (1 - 2a),  B_j = a m_j,  with m_j the Thomas pivots (see gp_api.cu).
 struct SweepParams {
   void* psi;             // field read by the sweep, layout [nz][ny][pitch]
-  void* out;             // field written (== psi except for the FP32 y / z sweeps)
+  void* out;             // field written (== psi except for the FP32 y / z sweeps, 2D: x / y)
   int nx, ny, nz;
   int pitch;             // row pitch of the field in elements
   int n;                 // line length along the swept axis
@@ -110,7 +110,7 @@ struct SweepParams {
   const void* vz;
   double dt, g;
   const double* scale;   // pending renormalisation factor, applied on load
-  // fused norm (z sweep, imaginary time only)
+  // fused norm (z sweep, or the y sweep of a 2D solve; imaginary time only)
   double* partials;
   unsigned int* counter;
   double* scale_out;
@@ -118,7 +118,8 @@ struct SweepParams {
   // per-block partials (norm_blocks of them) and sets *scale_state = 1; the next x
   // sweep (every block, the same fixed order) sums them into the factor it applies,
   // and any other reader of the factor first runs k_resolve_scale
-  int norm_defer;        // z: store partials only; x: take the factor from the partials
+  int plane_norm;        // y sweep of a 2D real field: the norm is summed there
+  int norm_defer;        // z (2D: y): store partials only; x: take the factor from the partials
   int norm_blocks;       // blocks of the z sweep (partials to sum)
   int norm_copies;       // z stores norm_copies copies of its partials (copy c at c norm_blocks);
                          // x block b reads copy b mod norm_copies: fewer readers per L2 line
@@ -210,15 +211,16 @@ cudaError_t x_band_prepare(int w, bool complex_field, bool grouped, size_t smem,
                            int* blocks_per_sm);
 cudaError_t launch_sweep_x_band(const SweepParams& p, bool complex_field, int grid,
                                 cudaStream_t st);
-// FP32 banded x sweep with the row in registers (rows of nx = 8 m <= 256, W in {3, 5}):
+// FP32 banded x sweep with the row in registers (real rows of nx = 8 m <= 256, W in {3, 5};
+// plane: a 2D solve, where x does not work in place):
 // blocks of kXRegWarps warps, no shared memory; band_rows rows per warp.
 bool x_reg_fits(int nx, int w);
-cudaError_t x_reg_prepare(int w, bool complex_field, int* blocks_per_sm);
-cudaError_t launch_sweep_x_reg(const SweepParams& p, bool complex_field, int grid, cudaStream_t st);
+cudaError_t x_reg_prepare(int w, bool plane, int* blocks_per_sm);
+cudaError_t launch_sweep_x_reg(const SweepParams& p, int grid, cudaStream_t st);
 // FP32 banded y / z sweeps (out of place like the streaming ones), blocks of 128 threads.
 cudaError_t launch_sweep_band_line(int axis, const SweepParams& p, bool complex_field, int grid,
                                    cudaStream_t st);
-int band_line_blocks_per_sm(int axis, bool complex_field, int w, bool cp);
+int band_line_blocks_per_sm(int axis, bool complex_field, bool norm, int w, bool cp);
 // Batched FP32 banded sweeps over the slots of a pool (one launch per direction
 // and mode): x on kBandWarps-warp blocks with dynamic shared memory
 // batch_x_smem(); y / z on blocks of 128 threads.  w is the launch half-width.

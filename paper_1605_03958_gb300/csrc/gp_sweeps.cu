@@ -701,6 +701,7 @@ __device__ __forceinline__ float2 shfl_down_e(float2 v, int d) {
 // stages of G row slots of slot_elems elements each.
 template <class E> struct XRows {
   E* field;
+  E* out;                // where the rows go (the field itself, or another buffer of its layout)
   const float4* fx;      // trap factors along x, [pitch] (16-byte vectors)
   const E* fyz;          // trap factor per row
   const E* wt;           // w_{k-W}, k = 0 .. 2W (centre as w_0 - 1)
@@ -848,7 +849,7 @@ __device__ __forceinline__ void x_band_rows(const XRows<typename Field<R, CPLX>:
         for (int k = 1; k <= W; ++k) acc = F::chain(wt[k], F::add(win[c - k], win[c + k]), acc);
         o[e] = F::add(win[c], acc);
       }
-      E* grow = field + (size_t)(gr0 + r) * pitch;
+      E* grow = a.out + (size_t)(gr0 + r) * pitch;
       if (x0 + EPT <= nx) {
         *reinterpret_cast<float4*>(grow + x0) = ov;
       } else {
@@ -911,7 +912,7 @@ __device__ __forceinline__ void x_band_rows_single(const XRows<typename Field<R,
   const bool pw = a.pw != 0;
   const E* fyz = a.fyz + a.row0;
   E f_next = fyz[0];
-  E* grow = field + (size_t)a.row0 * pitch;   // row i's output
+  E* grow = a.out + (size_t)a.row0 * pitch;   // row i's output
   int st = 0;
   uint32_t phase = 0;
 
@@ -1045,6 +1046,7 @@ __global__ void __launch_bounds__(32 * kBandWarps) k_sweep_x_band(const __grid_c
   if (nrow == 0) return;
   XRows<E> a;
   a.field = static_cast<E*>(p.psi);
+  a.out = static_cast<E*>(p.out);
   a.fx = static_cast<const float4*>(p.band_fx);
   a.fyz = static_cast<const E*>(p.band_fyz);
   a.wt = reinterpret_cast<const E*>(p.band_wt);
@@ -1076,7 +1078,7 @@ __global__ void __launch_bounds__(32 * kBandWarps) k_sweep_x_band(const __grid_c
 // shared memory, copies or waits: the instructions per point are the arithmetic plus
 // a few shuffles, which is what bounds the copy-fed kernel above.  Each warp works on
 // a_rows consecutive rows; every warp of the launch is resident at once.
-template <bool CPLX, int W>
+template <bool CPLX, int W, bool PLANE>
 __global__ void __launch_bounds__(32 * kXRegWarps) k_sweep_x_reg(const __grid_constant__ SweepParams p) {
   using F = Field<float, CPLX>;
   using E = typename F::E;
@@ -1110,6 +1112,7 @@ __global__ void __launch_bounds__(32 * kXRegWarps) k_sweep_x_reg(const __grid_co
   const float dtg = p.band_dtg;
   const bool pw = p.pw != 0;
   E* field = static_cast<E*>(p.psi);
+  E* out = PLANE ? static_cast<E*>(p.out) : field;   // (a run-time choice in 3D cost 0.3 us per step)
   const E* fyz = static_cast<const E*>(p.band_fyz);
   const long long nel = nrows * pitch;   // field elements (bounds checks)
   auto load_row = [&](long long r, float4 (&buf)[VPL]) {
@@ -1166,7 +1169,7 @@ __global__ void __launch_bounds__(32 * kXRegWarps) k_sweep_x_reg(const __grid_co
       o[e] = F::add(v[e], acc);
     }
     if (act && GP_IN(r * pitch + x0 + 7, nel, p.status)) {
-      float4* dst = reinterpret_cast<float4*>(field + (size_t)r * pitch + x0);
+      float4* dst = reinterpret_cast<float4*>(out + (size_t)r * pitch + x0);
 #pragma unroll
       for (int q = 0; q < VPL; ++q) dst[q] = *reinterpret_cast<const float4*>(&o[q * EPT]);
     }
@@ -1227,7 +1230,7 @@ __global__ void __launch_bounds__(32 * kBatchXWarps) k_batch_x_band(const __grid
   const XItem it = static_cast<const XItem*>(b.items)[w];
   const SlotDesc& d = b.slots[it.slot];
   XRows<E> a;
-  a.field = static_cast<E*>(d.field);
+  a.field = a.out = static_cast<E*>(d.field);
   a.fx = static_cast<const float4*>(d.fx);
   a.fyz = static_cast<const E*>(d.fyz);
   a.wt = reinterpret_cast<const E*>(d.wt[0]) + (kBandHalfMax - W);
@@ -1840,24 +1843,24 @@ cudaError_t x_band_prepare(int w, bool complex_field, bool grouped, size_t smem,
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, 32 * kBandWarps, smem);
 }
 
-static void (*x_reg_kernel_for(int w, bool cplx))(SweepParams) {
+static void (*x_reg_kernel_for(int w, bool plane))(SweepParams) {
   switch (w) {
-    case 3: return cplx ? k_sweep_x_reg<true, 3> : k_sweep_x_reg<false, 3>;
-    case 5: return cplx ? k_sweep_x_reg<true, 5> : k_sweep_x_reg<false, 5>;
+    case 3: return plane ? k_sweep_x_reg<false, 3, true> : k_sweep_x_reg<false, 3, false>;
+    case 5: return plane ? k_sweep_x_reg<false, 5, true> : k_sweep_x_reg<false, 5, false>;
     default: return nullptr;
   }
 }
 
 bool x_reg_fits(int nx, int w) { return nx % 8 == 0 && nx <= 256 && (w == 3 || w == 5); }
 
-cudaError_t x_reg_prepare(int w, bool complex_field, int* blocks_per_sm) {
-  void (*k)(SweepParams) = x_reg_kernel_for(w, complex_field);
+cudaError_t x_reg_prepare(int w, bool plane, int* blocks_per_sm) {
+  void (*k)(SweepParams) = x_reg_kernel_for(w, plane);
   if (!k) return cudaErrorInvalidValue;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, 32 * kXRegWarps, 0);
 }
 
-cudaError_t launch_sweep_x_reg(const SweepParams& p, bool complex_field, int grid, cudaStream_t st) {
-  void (*k)(SweepParams) = x_reg_kernel_for(p.band_w, complex_field);
+cudaError_t launch_sweep_x_reg(const SweepParams& p, int grid, cudaStream_t st) {
+  void (*k)(SweepParams) = x_reg_kernel_for(p.band_w, p.nz == 1);
   if (!k) return cudaErrorInvalidValue;
   return launch_pdl(k, grid, 32 * kXRegWarps, 0, st, p);
 }
@@ -1873,7 +1876,8 @@ cudaError_t launch_sweep_x_band(const SweepParams& p, bool complex_field, int gr
 static size_t band_line_smem(int W, bool cp) { return cp ? (size_t)128 * 2 * (2 * W + 1) * 16 : 0; }
 
 using SweepKernel = void (*)(SweepParams);
-template <int W, bool CP> static SweepKernel band_line_kernel(int axis, bool cplx) {
+template <int W, bool CP> static SweepKernel band_line_kernel(int axis, bool cplx, bool norm) {
+  if (axis == 1 && norm && !cplx) return k_sweep_band_line<float, false, 1, true, W, CP>;
   if (axis == 1)
     return cplx ? k_sweep_band_line<float, true, 1, false, W, CP> : k_sweep_band_line<float, false, 1, false, W, CP>;
   return cplx ? k_sweep_band_line<float, true, 2, false, W, CP> : k_sweep_band_line<float, false, 2, true, W, CP>;
@@ -1883,12 +1887,13 @@ template <int W>
 static cudaError_t launch_band_line_W(int axis, const SweepParams& p, bool cplx, int grid,
                                      cudaStream_t st) {
   const bool cp = p.band_cp != 0;
-  void (*k)(SweepParams) = cp ? band_line_kernel<W, true>(axis, cplx) : band_line_kernel<W, false>(axis, cplx);
+  const bool norm = p.plane_norm != 0;
+  void (*k)(SweepParams) = cp ? band_line_kernel<W, true>(axis, cplx, norm) : band_line_kernel<W, false>(axis, cplx, norm);
   return launch_pdl(k, grid, 128, band_line_smem(W, cp), st, p);
 }
 
-template <int W> static int band_line_blocks_per_sm_W(int axis, bool cplx, bool cp) {
-  void (*k)(SweepParams) = cp ? band_line_kernel<W, true>(axis, cplx) : band_line_kernel<W, false>(axis, cplx);
+template <int W> static int band_line_blocks_per_sm_W(int axis, bool cplx, bool norm, bool cp) {
+  void (*k)(SweepParams) = cp ? band_line_kernel<W, true>(axis, cplx, norm) : band_line_kernel<W, false>(axis, cplx, norm);
   const size_t smem = band_line_smem(W, cp);
   if (smem > 48 * 1024 &&
       cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
@@ -1900,11 +1905,11 @@ template <int W> static int band_line_blocks_per_sm_W(int axis, bool cplx, bool 
   return b;
 }
 
-int band_line_blocks_per_sm(int axis, bool complex_field, int w, bool cp) {
+int band_line_blocks_per_sm(int axis, bool complex_field, bool norm, int w, bool cp) {
   switch (w) {
-    case 3: return band_line_blocks_per_sm_W<3>(axis, complex_field, cp);
-    case 5: return band_line_blocks_per_sm_W<5>(axis, complex_field, cp);
-    case 8: return band_line_blocks_per_sm_W<8>(axis, complex_field, cp);
+    case 3: return band_line_blocks_per_sm_W<3>(axis, complex_field, norm, cp);
+    case 5: return band_line_blocks_per_sm_W<5>(axis, complex_field, norm, cp);
+    case 8: return band_line_blocks_per_sm_W<8>(axis, complex_field, norm, cp);
     default: return 0;
   }
 }

@@ -1034,8 +1034,9 @@ static size_t inc64_x_smem(unsigned threads, int X) {
 
 // shared-memory limit of the increment kernels (blocks of kIncThreads)
 static cudaError_t inc64_prepare() {
-  void (*const k[4])(SweepParams) = {k_sweep_inc64<false, 1, false>, k_sweep_inc64<false, 2, true>,
-                                     k_sweep_inc64<true, 1, false>, k_sweep_inc64<true, 2, false>};
+  void (*const k[5])(SweepParams) = {k_sweep_inc64<false, 1, false>, k_sweep_inc64<false, 1, true>,
+                                     k_sweep_inc64<false, 2, true>, k_sweep_inc64<true, 1, false>,
+                                     k_sweep_inc64<true, 2, false>};
   for (auto f : k) {
     const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)((kIncL + 2) * kIncThreads * sizeof(float4)));
@@ -1084,6 +1085,7 @@ cudaError_t launch_inc64(int axis, const SweepParams& p, bool complex_field, cud
     return complex_field ? cudaLaunchKernelEx(&cfg, k_sweep_xinc64<true>, q)
                          : cudaLaunchKernelEx(&cfg, k_sweep_xinc64<false>, q);
   }
+  if (axis == 1 && p.plane_norm) return cudaLaunchKernelEx(&cfg, k_sweep_inc64<false, 1, true>, p);
   if (axis == 1)
     return complex_field ? cudaLaunchKernelEx(&cfg, k_sweep_inc64<true, 1, false>, p)
                          : cudaLaunchKernelEx(&cfg, k_sweep_inc64<false, 1, false>, p);

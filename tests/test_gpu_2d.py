@@ -70,3 +70,27 @@ def test_2d_strang(P, orc):
     s.step_imag(30)
     assert np.max(np.abs(s.get_psi() - ref)) <= 1e-10
     s.close()
+
+
+@pytest.mark.parametrize("shape", [(96, 80), (37, 53), (300, 12), (128, 9), (1000, 40)])
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+@pytest.mark.parametrize("scheme", ["lie", "strang"])
+def test_2d_norm_fused_into_the_y_sweep(P, orc, shape, prec, scheme):
+    """x into the staging area, y back with the norm: single-step calls (a graph), runs and
+    reads between them against the oracle's run.  Tolerances: FP32 as the short 3D runs
+    (44 roundings of 2^-24 per step and point, a random walk), FP64 64 steps 2^-53."""
+    p = p2(orc, *shape)
+    n = 6
+    ref = (orc.step_imag_strang if scheme == "strang" else orc.step_imag)(p, orc.init_gaussian(p), n)
+    s = solver(P, p, prec)
+    s.set_splitting(scheme)
+    s.init_gaussian()
+    s.step_imag(1)
+    s.step_imag(3)
+    assert abs(s.observables()["norm"] - 1.0) <= (1e-6 if prec == "f32" else 1e-13)
+    s.step_imag(1)
+    s.sync()
+    s.step_imag(1)
+    tol = n * np.sqrt(44) * 2.0 ** -24 if prec == "f32" else 64 * n * 2.0 ** -53
+    assert np.max(np.abs(s.get_psi() - ref)) <= tol * np.max(np.abs(ref))
+    s.close()
