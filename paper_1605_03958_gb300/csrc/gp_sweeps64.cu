@@ -517,7 +517,7 @@ __device__ __forceinline__ void inc_segment(const IncRho<CPLX>& rho, float4* slo
   int tmax = 0;
   // noise: somewhere sampled, the second difference is opposite in sign to v and larger
   // than the values (complex: the moduli) around it and than least
-  bool fp64 = false;
+  bool noisy = false;
   {
     const double2 v0 = get_d2(slot);
     Three a = split3(before.x, before.y, &tmax), b = split3(v0.x, v0.y, &tmax);
@@ -531,15 +531,19 @@ __device__ __forceinline__ void inc_segment(const IncRho<CPLX>& rho, float4* slo
         float lx = fmaxf(least, fmaxf(fabsf(a.h.x), fmaxf(fabsf(b.h.x), fabsf(c.h.x))));
         float ly = fmaxf(least, fmaxf(fabsf(a.h.y), fmaxf(fabsf(b.h.y), fabsf(c.h.y))));
         if (CPLX) lx = ly = fmaxf(lx, ly);
-        fp64 = fp64 || (fabsf(s.h.x) > lx && s.h.x * b.h.x < 0.f) ||
+        noisy = noisy || (fabsf(s.h.x) > lx && s.h.x * b.h.x < 0.f) ||
                (fabsf(s.h.y) > ly && s.h.y * b.h.y < 0.f);
       }
       a = b;
       b = c;
     }
   }
-  fp64 = fp64 || tmax >= kSplitTooBig;
-  if (!__syncthreads_or(on && fp64)) {
+  // values out of range, or noise at half the segments of a warp: the block computes in FP64
+  // (one noisy segment is not enough: a field with fine structure here and there keeps its
+  // accuracy, and most blocks of a turbulent field would go: 101 x 77 x 53 complex, 20
+  // steps late in a run 2281 us, with half a warp 1351)
+  const bool noise = __popc(__ballot_sync(0xffffffffu, on && noisy)) >= 16;
+  if (!__syncthreads_or(noise || (on && tmax >= kSplitTooBig))) {
     // carry out to the next segment: the tail of s; the first segment also starts itself
     put_two(carry, inc_carry(rho, [&](int k) { return get_two(slot + (kIncL - 1 - k) * TS); }));
     Prod pr = prod_zero();
