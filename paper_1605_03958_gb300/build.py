@@ -18,7 +18,7 @@ LIB = os.path.join(OUT_DIR, "libgp_sscn.so")
 # the same library with the kernels' bounds checks on (-DGP_CHECK): an index outside
 # its buffer records a status the host reports as GP_ERR_BOUNDS instead of faulting
 LIB_CHECK = os.path.join(OUT_DIR, "libgp_sscn_check.so")
-SOURCES = ["gp_api.cu", "gp_sweeps.cu", "gp_sweeps64.cu", "gp_reduce.cu", "gp_noalloc.cu",
+SOURCES = ["gp_api.cu", "gp_sweeps.cu", "gp_sweeps_tile.cu", "gp_sweeps64.cu", "gp_reduce.cu", "gp_noalloc.cu",
            "gp_batch.cu"]
 HEADERS = ["gp_device.cuh", "gp_split.cuh", "gp_internal.h", "gp_arena.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -614,6 +614,19 @@ void fill_sweep_params(gp_solver* s) {
         }
         q.band_seg = best_seg;
         s->fast_grid[m][a] = (int)blocks;
+        // over shared-memory tiles (a norm partial per block must fit there too): fields of up
+        // to 40 MB, which both buffers leave in L2, and the real y sweep of any size; beyond,
+        // a run per thread was as fast or faster (complex z 240x200x160, 61 MB: 21.6 against
+        // 22.6 us; 512x400x320 y / z 160 / 158 against 164 / 162; real y 300x240x200, 58 MB:
+        // tiles 22.9 against 25.5 us, 512x400x320 84.2 against 84.4)
+        const bool norm = m == 0 && (a == 2 || p.nz == 1);
+        const bool fits = s->L.field_bytes / (m == 0 ? 2 : 1) <= (size_t)40 << 20;
+        const long long tiles = forced > 0 || !q.band_cp || !(fits || (m == 0 && a == 1))
+                                    ? 0 : gpk::band_tile_setup(a, &q, m == 1);
+        if (tiles > 0 && (!norm || tiles <= (long long)s->L.npartials)) {
+          s->fast_grid[m][a] = (int)tiles;
+          q.band_cp = 2;
+        }
       }
     }
   // 2D, banded x and y sweeps: x goes from the field to the staging area and y back, so
@@ -955,6 +968,8 @@ template <class R> int run_sweep(gp_solver* s, int axis) {
     e = gpk::launch_sweep_x_reg(q, s->fast_grid[m][0], s->stream);
   else if (axis == 0 && q.band_w)
     e = gpk::launch_sweep_x_band(q, m == 1, s->fast_grid[m][0], s->stream);
+  else if (q.band_w && q.band_cp == 2)
+    e = gpk::launch_band_tile(axis, q, m == 1, s->fast_grid[m][axis], s->stream);
   else if (q.band_w)
     e = gpk::launch_sweep_band_line(axis, q, m == 1, s->fast_grid[m][axis], s->stream);
   else if (q.trunc)

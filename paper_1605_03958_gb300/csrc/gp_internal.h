@@ -90,9 +90,11 @@ struct SweepParams {
   int band_stages;       // x: groups of rows in flight per warp
   int band_group;        // x: rows per group (worked on together by the warp's lanes)
   int band_seg;          // y / z: points per line segment (a multiple of 2 band_w + 1)
-  int band_cp;           // y / z: 1 = next turn's inputs copied to shared memory ahead (cp.async)
+  int band_cp;           // y / z: 2 = shared-memory tiles (k_band_tile), 1 = a run per thread, next turn's
+                         // inputs copied to shared memory ahead (cp.async), 0 = in registers
   int band_reg;          // x: 1 = the row in registers (k_sweep_x_reg)
   float band_dtg;        // x: dt g in FP32
+  int tile_run, tile_cols;   // y / z over tiles (gp_sweeps_tile.cu): points per run, vectors per block
   // FP64 increment sweeps (gp_sweeps64.cu): decay factor rho of the CN solve's two
   // one-sided recursions, rho + 1/rho = (1+2a)/a, in FP64 (re, im) and as the FP32 pairs
   // (re hi, re lo, im hi, im lo); 16-byte vectors per block row and segments per line
@@ -221,6 +223,10 @@ cudaError_t launch_sweep_x_reg(const SweepParams& p, int grid, cudaStream_t st);
 cudaError_t launch_sweep_band_line(int axis, const SweepParams& p, bool complex_field, int grid,
                                    cudaStream_t st);
 int band_line_blocks_per_sm(int axis, bool complex_field, bool norm, int w, bool cp);
+// FP32 banded sweeps over shared-memory tiles (gp_sweeps_tile.cu): set-up (fills p's tile_*
+// fields; returns the blocks of the launch, 0: not possible) and launch.
+long long band_tile_setup(int axis, SweepParams* p, bool complex_field);
+cudaError_t launch_band_tile(int axis, const SweepParams& p, bool complex_field, int grid, cudaStream_t st);
 // Batched FP32 banded sweeps over the slots of a pool (one launch per direction
 // and mode): x on kBandWarps-warp blocks with dynamic shared memory
 // batch_x_smem(); y / z on blocks of 128 threads.  w is the launch half-width.
