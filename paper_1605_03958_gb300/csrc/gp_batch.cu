@@ -1,7 +1,7 @@
 // gp_batch.cu -- pools of resident FP32 solves stepped together (batched uneven
 // solves and the serving loop): a device arena with a first-fit allocator, per-slot
 // tables and descriptors, packed work lists (rows of every x line; blocks of every
-// y / z line segment), one batched launch per sweep direction and mode, the step
+// slot's y / z tiles), one batched launch per sweep direction and mode, the step
 // captured as a CUDA graph, per-slot observables and field I/O, and an autotuner over
 // the launch shapes.  Every slot runs the same SSCN step as a single FP32 solver
 // (paper, program summary: "Solution method") with the banded line operators of
@@ -45,7 +45,7 @@ struct SlotGeom {
   size_t field_bytes = 0;      // sized for the complex field
   size_t off_field = 0, off_staging = 0, off_fx[2] = {}, off_fyz[2] = {}, off_otab = 0;
   size_t off_scal = 0, off_partials = 0, total = 0;
-  int max_blocks_z = 0;        // z blocks of the slot at the shortest segment
+  int max_blocks_z = 0;        // z blocks of the slot that its partials area takes
 };
 
 void slot_geometry(const gp_params& p, SlotGeom* G) {
@@ -53,14 +53,13 @@ void slot_geometry(const gp_params& p, SlotGeom* G) {
   G->pitch[0] = (int)align_up((size_t)p.nx, 4);
   G->pitch[1] = (int)align_up((size_t)p.nx, 2);
   G->field_bytes = std::max((size_t)G->pitch[0] * 4, (size_t)G->pitch[1] * 8) * rows;
-  // z blocks at the shortest segment (one turn of the smallest ring, 7 points)
+  // z blocks at the shortest run (one turn of the smallest ring, 7 points)
   int mb = 0;
   for (int m = 0; m < 2; ++m) {
     const long long cols = (long long)((p.nx + (m ? 1 : 3)) / (m ? 2 : 4)) * p.ny;
     const long long nseg = (p.nz + 6) / 7;
     mb = std::max<int>(mb, (int)((cols * nseg + 127) / 128));
   }
-  G->max_blocks_z = mb;
   size_t off = 0;
   G->off_field = off;
   off = align_up(off + G->field_bytes, kAlign);
@@ -78,6 +77,7 @@ void slot_geometry(const gp_params& p, SlotGeom* G) {
   off = align_up(off + 64, kAlign);
   G->off_partials = off;
   off = align_up(off + (size_t)mb * 8, kAlign);
+  G->max_blocks_z = (int)((off - G->off_partials) / 8);
   G->total = off;
 }
 
@@ -124,6 +124,7 @@ struct gp_pool {
   int wl[2][3] = {};           // launch half-width per mode and axis
   int slot_elems[2] = {};      // x: shared-memory row slot per mode
   size_t x_smem[2] = {};
+  size_t tile_smem[2][3] = {};   // y / z: shared memory of a block per mode and axis
   int x_stages_used[2] = {2, 2};
   bool x_reg[2] = {false, false};    // x sweep with rows in registers for the mode's slots
   int x_group_max[2] = {1, 1};
@@ -284,6 +285,7 @@ int rebuild(gp_pool* P) {
     P->live_mode[m] = 0;
     P->slot_elems[m] = 0;
     for (int a = 0; a < 3; ++a) P->wl[m][a] = 0;
+    P->tile_smem[m][1] = P->tile_smem[m][2] = 0;
   }
   for (int i = 0; i < ns; ++i) {
     const Slot& S = P->slots[i];
@@ -312,7 +314,17 @@ int rebuild(gp_pool* P) {
     d.ny = S.prm.ny;
     d.nz = S.prm.nz;
     d.pitch = S.G.pitch[m];
-    for (int a = 1; a < 3; ++a) d.seg[a] = P->seg_turns * (2 * P->wl[m][a] + 1);
+    for (int a = 1; a < 3; ++a) {
+      const int n = a == 1 ? d.ny : d.nz;
+      int turns = P->seg_turns;
+      gpk::batch_tile_shape(n, P->wl[m][a], turns, m == 0 && a == 2, &d.tile_runs[a], &d.tile_run[a]);
+      // one norm partial per z block must fit the slot's area (a single run always does)
+      while (m == 0 && a == 2 && turns > 1 &&
+             gpk::batch_tile_blocks(d.nx, d.ny, n, d.tile_runs[a], d.tile_run[a], false) > S.G.max_blocks_z) {
+        turns = std::min(turns, 3) - 1;
+        gpk::batch_tile_shape(n, P->wl[m][a], turns, m == 0 && a == 2, &d.tile_runs[a], &d.tile_run[a]);
+      }
+    }
     d.dtg = (float)(S.prm.dt * S.g);
     d.dV = S.prm.dx * S.prm.dy * S.prm.dz;
     std::memcpy(d.wt, S.wt[m], sizeof d.wt);
@@ -388,13 +400,12 @@ int rebuild(gp_pool* P) {
         it.pad = 0;
         xi.push_back(it);
       }
-      const int ept = cplx ? 2 : 4;
       for (int a = 1; a < 3; ++a) {
-        const int n = a == 1 ? S.prm.ny : S.prm.nz;
-        const long long cols = (long long)((S.prm.nx + ept - 1) / ept) * (a == 1 ? S.prm.nz : S.prm.ny);
-        const int seg = P->seg_turns * (2 * P->wl[m][a] + 1);
-        const long long nb = (cols * ((n + seg - 1) / seg) + 127) / 128;
-        if (a == 2 && nb > S.G.max_blocks_z) return pfail(P, GP_ERR_ARG, "z blocks exceed the slot's partials");
+        const SlotDesc& d = P->h_desc[i];
+        const int n = a == 1 ? d.ny : d.nz, nother = a == 1 ? d.nz : d.ny;
+        const long long nb = gpk::batch_tile_blocks(d.nx, nother, n, d.tile_runs[a], d.tile_run[a], cplx);
+        P->tile_smem[m][a] = std::max(P->tile_smem[m][a], gpk::batch_tile_smem(d.tile_runs[a], d.tile_run[a], P->wl[m][a]));
+        if (!cplx && a == 2 && nb > S.G.max_blocks_z) return pfail(P, GP_ERR_ARG, "z blocks exceed the slot's partials");
         for (long long q = 0; q < nb; ++q) {
           LineBlock l;
           l.slot = i;
@@ -440,7 +451,8 @@ int launch_step(gp_pool* P) {
       const int xw = b.x_reg ? gpk::kXRegWarps : gpk::kBatchXWarps;
       const int grid = a == 0 ? (b.nitems + xw - 1) / xw : b.nitems;
       const cudaError_t e = gpk::launch_batch_sweep(a, P->wl[m][a], b, m == 1, grid,
-                                                    a == 0 && !b.x_reg ? P->x_smem[m] : 0, P->stream);
+                                                    a > 0 ? P->tile_smem[m][a] : b.x_reg ? 0 : P->x_smem[m],
+                                                    P->stream);
       if (e != cudaSuccess) return pcuda(P, e, "batched sweep launch");
     }
   }

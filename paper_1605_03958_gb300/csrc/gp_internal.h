@@ -146,7 +146,7 @@ struct SlotDesc {
   double* partials;       // z-sweep norm partials, one per z block of the slot
   unsigned int* counter;  // z blocks of the slot finished (reset by the last)
   int nx, ny, nz, pitch;
-  int seg[3];             // y / z: segment length in points
+  int tile_runs[3], tile_run[3];   // y / z: runs per block, points per run
   float dtg;              // dt g
   double dV;
   // banded weights per axis, w_{k-8}, k = 0 .. 16 (centre as w_0 - 1; complex:
@@ -229,7 +229,7 @@ long long band_tile_setup(int axis, SweepParams* p, bool complex_field);
 cudaError_t launch_band_tile(int axis, const SweepParams& p, bool complex_field, int grid, cudaStream_t st);
 // Batched FP32 banded sweeps over the slots of a pool (one launch per direction
 // and mode): x on kBandWarps-warp blocks with dynamic shared memory
-// batch_x_smem(); y / z on blocks of 128 threads.  w is the launch half-width.
+// batch_x_smem(); y / z on the tiles below.  w is the launch half-width.
 size_t batch_x_smem(int stages, int group_max, int slot_elems, bool complex_field);
 // Rows per group of the banded x sweep for rows of nx points (ept per 16-byte vector):
 // the cost model's best G in 1..8 whose stages fit warp_budget bytes of row slots.
@@ -237,6 +237,12 @@ int x_band_group(int nx, int ept, int stages, size_t slot_bytes, size_t warp_bud
 cudaError_t batch_prepare(int w, bool complex_field, size_t x_smem, int* x_blocks_per_sm);
 cudaError_t launch_batch_sweep(int axis, int w, const BatchArgs& b, bool complex_field, int grid,
                                size_t smem, cudaStream_t st);
+// Batched y / z sweeps over shared-memory tiles (gp_sweeps_tile.cu): runs per block and points
+// per run of a line of n points, blocks of a slot, shared memory of a block, launch.
+void batch_tile_shape(int n, int w, int turns, bool norm, int* runs, int* run);
+long long batch_tile_blocks(int nx, int nother, int n, int runs, int run, bool complex_field);
+size_t batch_tile_smem(int runs, int run, int w);
+cudaError_t launch_batch_tile(int axis, int w, const BatchArgs& b, bool complex_field, size_t smem, cudaStream_t st);
 // Batched x sweep with rows in registers (slots of nx = 16 m <= 512 real or 8 m <= 256
 // complex points, W in {3, 5}): whether a slot fits, and the resident blocks of
 // kXRegWarps warps per SM.

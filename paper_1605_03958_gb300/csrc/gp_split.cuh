@@ -404,4 +404,64 @@ GP_HD double to_double(float h, float l, int k) {
   return from_words((uint32_t)(w >> 32), (uint32_t)w);
 }
 
+#ifdef __CUDACC__
+// The banded operator (gp_sweeps.cu) on two lanes at a time: two points of a real line, or
+// the parts of one complex point, its products as two real sums, A = sum w.re s and
+// B = sum w.im s, joined at the end (4 W + 5 instructions; 8 W + 6 as complex products).
+template <bool CPLX, int W> struct BandTaps {
+  float2 wr[W + 1], wi[CPLX ? W + 1 : 1];
+  __device__ __forceinline__ explicit BandTaps(const float* wt) {   // centre first
+#pragma unroll
+    for (int k = 0; k <= W; ++k) {
+      wr[k] = f2(CPLX ? wt[2 * (W + k)] : wt[W + k]);
+      if constexpr (CPLX) wi[k] = f2(wt[2 * (W + k) + 1]);
+    }
+  }
+  // at(k): the value k points along the line (a float2 of the vector)
+  template <class AT> __device__ __forceinline__ float2 operator()(AT at) const {
+    const float2 c = at(0);
+    float2 a = mul2(wr[0], c);
+    if constexpr (CPLX) {
+      float2 b = mul2(wi[0], c);
+#pragma unroll
+      for (int k = 1; k <= W; ++k) {
+        const float2 s = add2(at(-k), at(k));
+        a = fma2(wr[k], s, a);
+        b = fma2(wi[k], s, b);
+      }
+      return add2(c, f2(a.x - b.y, a.y + b.x));
+    } else {
+#pragma unroll
+      for (int k = 1; k <= W; ++k) a = fma2(wr[k], add2(at(-k), at(k)), a);
+      return add2(c, a);
+    }
+  }
+};
+// The same operator with the complex products' roundings of Field::chain (gp_device.cuh),
+// each tap added to the result before it; real lines: as BandTaps.
+template <bool CPLX, int W> struct BandChain : BandTaps<CPLX, W> {
+  using BandTaps<CPLX, W>::wr;
+  using BandTaps<CPLX, W>::wi;
+  __device__ __forceinline__ explicit BandChain(const float* wt) : BandTaps<CPLX, W>(wt) {
+    if constexpr (CPLX)
+#pragma unroll
+      for (int k = 0; k <= W; ++k) wi[k].x = -wi[k].x;
+  }
+  template <class AT> __device__ __forceinline__ float2 operator()(AT at) const {
+    if constexpr (CPLX) {
+      const float2 c = at(0);
+      float2 a = fma2(wr[0], c, mul2(wi[0], f2(c.y, c.x)));
+#pragma unroll
+      for (int k = 1; k <= W; ++k) {
+        const float2 s = add2(at(-k), at(k));
+        a = fma2(wr[k], s, fma2(wi[k], f2(s.y, s.x), a));
+      }
+      return add2(c, a);
+    } else {
+      return BandTaps<CPLX, W>::operator()(at);
+    }
+  }
+};
+#endif
+
 }  // namespace gpk
