@@ -273,6 +273,11 @@ bool band_prefetch() {
   const char* v = std::getenv("GP_BAND_PREFETCH");
   return !(v && std::strcmp(v, "0") == 0);
 }
+// GP_XY=0 keeps the x and y sweeps of small grids separate (A/B measurements).
+bool xy_enabled() {
+  const char* v = std::getenv("GP_XY");
+  return !(v && std::strcmp(v, "0") == 0);
+}
 bool force_stream() {
   const char* v = std::getenv("GP_SWEEP_KERNELS");
   return v && (std::strcmp(v, "stream") == 0 || std::strcmp(v, "stream_x") == 0);
@@ -323,6 +328,7 @@ struct gp_solver {
   unsigned int* counters = nullptr;  // [0] sweeps, [1] reductions
   double* obs = nullptr;
   SweepParams sp[2][3];
+  SweepParams sp_xy[2] = {};         // x and y in one pass (xy_parts > 0)
   int head[2][3] = {};               // see SweepParams::head
   int trunc[2][3] = {};              // FP32 fast sweeps: truncation depth, 0 = use the tile kernel
   int fast_grid[2][3] = {};          // blocks of the fast sweeps (x band: persistent grid)
@@ -488,6 +494,7 @@ void fill_sweep_params(gp_solver* s) {
       q.scale = s->scale;
       // FP32 field in imaginary time: the renormalisation factor is dithered per step
       q.step_ctr = (m == 0 && s->L.rbytes == 4) ? s->step_ctr : nullptr;
+      q.step_count = q.step_ctr && a == 1 ? 1 : 0;
       q.partials = s->partials;
       q.counter = s->counters;
       q.scale_out = s->scale;
@@ -636,6 +643,16 @@ void fill_sweep_params(gp_solver* s) {
       s->sp[m][0].out = s->sp[m][1].psi = s->staging;
       s->sp[m][1].out = s->field;
     }
+  // small 3D grids, banded sweeps of one half-width along x and y: both in one launch, from
+  // the field to the staging area
+  for (int m = 0; m < 2 && p.nz > 1 && x_reg_enabled(); ++m) {
+    SweepParams q = s->sp[m][0];
+    q.out = s->sp[m][1].out;
+    std::memcpy(q.band_wt_y, s->sp[m][1].band_wt, sizeof q.band_wt_y);
+    if (!xy_enabled() || q.band_w == 0 || q.band_w != s->band_w[m][1] || !gpk::band_xy_setup(&q, m == 1))
+      q.xy_parts = 0;
+    s->sp_xy[m] = q;
+  }
   // FP32 real field, banded x sweep and banded last sweep (z; 2D: y): the last sweep only
   // stores its norm partials and the next x sweep sums them (every block, in the same
   // order) into the factor it applies, instead of the last block summing them at the end;
@@ -649,6 +666,12 @@ void fill_sweep_params(gp_solver* s) {
     q.norm_copies = std::max(1, std::min(8, (int)(s->L.npartials / std::max(1, s->fast_grid[0][la]))));
     q.scale_state = s->scale_state;
   }
+  SweepParams& xy = s->sp_xy[0];
+  const SweepParams& x = s->sp[0][0];
+  xy.norm_defer = x.norm_defer;
+  xy.norm_blocks = x.norm_blocks;
+  xy.norm_copies = x.norm_copies;
+  xy.scale_state = x.scale_state;
 }
 
 template <class T> void put(std::vector<unsigned char>& buf, size_t off, const T& v) {
@@ -950,12 +973,25 @@ struct NvtxRange {
   ~NvtxRange() { nvtxRangePop(); }
 };
 
+// x and y in one pass: wherever set up, except while sweeps are timed one by one.
+bool xy_joined(const gp_solver* s) { return s->sp_xy[s->is_complex ? 1 : 0].xy_parts > 0 && !s->timing; }
+
+int run_xy(gp_solver* s) {
+  NvtxRange range("gp sweep xy");
+  const int m = s->is_complex ? 1 : 0;
+  SweepParams q = s->sp_xy[m];
+  if (s->kinetic_only) q.pw = 0;
+  const cudaError_t e = gpk::launch_band_xy(q, m == 1, s->stream);
+  return e == cudaSuccess ? GP_OK : cuda_fail(s, e, "sweep launch");
+}
+
 template <class R> int run_sweep(gp_solver* s, int axis) {
   static const char* const kNames[3] = {"gp sweep x", "gp sweep y", "gp sweep z"};
   NvtxRange range(kNames[axis]);
   const int m = s->is_complex ? 1 : 0;
   SweepParams q = s->sp[m][axis];
   if (axis == 0 && s->kinetic_only) q.pw = 0;
+  if (axis == 2 && xy_joined(s)) q.step_count = q.step_ctr ? 1 : 0;
   const size_t smem = s->L.geom[m][axis].smem;
   TimedLaunch tl{nullptr, nullptr, axis};
   if (s->timing) {
@@ -1015,7 +1051,8 @@ template <class R> int lie_step_direct(gp_solver* s) {
         }
         continue;
       }
-      const int rc = run_sweep<R>(s, a);
+      if (a == 1 && xy_joined(s)) continue;
+      const int rc = a == 0 && xy_joined(s) ? run_xy(s) : run_sweep<R>(s, a);
       if (rc != GP_OK) return rc;
     }
   }
@@ -1519,7 +1556,7 @@ int gp_set_g(gp_solver* s, double g) {
   for (int m = 0; m < 2; ++m)
     for (int a = 0; a < 3; ++a) {
       s->sp[m][a].g = g;
-      s->sp[m][a].band_dtg = (float)(s->sp[m][a].dt * g);
+      s->sp[m][a].band_dtg = s->sp_xy[m].band_dtg = (float)(s->sp[m][a].dt * g);
     }
   drop_step_graphs(s);   // they hold the old parameters
   return GP_OK;

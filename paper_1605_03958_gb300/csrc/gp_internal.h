@@ -95,6 +95,10 @@ struct SweepParams {
   int band_reg;          // x: 1 = the row in registers (k_sweep_x_reg)
   float band_dtg;        // x: dt g in FP32
   int tile_run, tile_cols;   // y / z over tiles (gp_sweeps_tile.cu): points per run, vectors per block
+  // x and y in one pass (gp_sweeps_tile.cu; in the x sweep's parameters, with the y sweep's
+  // out): rows per block, blocks per plane (0: not used), points per run, shared memory
+  int xy_rows, xy_parts, xy_run, xy_smem;
+  float band_wt_y[2 * 17];   // the y sweep's weights
   // FP64 increment sweeps (gp_sweeps64.cu): decay factor rho of the CN solve's two
   // one-sided recursions, rho + 1/rho = (1+2a)/a, in FP64 (re, im) and as the FP32 pairs
   // (re hi, re lo, im hi, im lo); 16-byte vectors per block row and segments per line
@@ -127,9 +131,10 @@ struct SweepParams {
                          // x block b reads copy b mod norm_copies: fewer readers per L2 line
   int* scale_state;      // 1: the factor is the partials' 1 / sqrt(sum dV)
   // FP32 field in imaginary time: the step counter behind the renormalisation factor's
-  // dither (step_dither in gp_device.cuh): the sweeps that apply the factor read it, the
-  // y sweep adds one; null otherwise (no dither)
+  // dither (step_dither in gp_device.cuh): the sweeps that apply the factor read it, a later
+  // sweep of the step (y, or z when x and y are one) adds one; null otherwise (no dither)
   unsigned int* step_ctr;
+  int step_count;        // 1: this sweep adds one
   int* status;
   double dV;
   long long ntiles;
@@ -227,6 +232,10 @@ int band_line_blocks_per_sm(int axis, bool complex_field, bool norm, int w, bool
 // fields; returns the blocks of the launch, 0: not possible) and launch.
 long long band_tile_setup(int axis, SweepParams* p, bool complex_field);
 cudaError_t launch_band_tile(int axis, const SweepParams& p, bool complex_field, int grid, cudaStream_t st);
+// x and y sweeps of a small 3D solve in one pass: set-up of the x sweep's parameters (band_* filled;
+// fills xy_*; false: not a grid for it) and launch.
+bool band_xy_setup(SweepParams* p, bool complex_field);
+cudaError_t launch_band_xy(const SweepParams& p, bool complex_field, cudaStream_t st);
 // Batched FP32 banded sweeps over the slots of a pool (one launch per direction
 // and mode): x on kBandWarps-warp blocks with dynamic shared memory
 // batch_x_smem(); y / z on the tiles below.  w is the launch half-width.

@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(32) k_sweep_y(const __grid_constant__ CUtensor
                                                 const SweepParams p) {
   pdl_begin();
   // the factor's dither (FP32, imaginary time): the step's x sweep has read the counter
-  if (p.step_ctr && blockIdx.x == 0 && threadIdx.x == 0) *p.step_ctr += 1;
+  if (p.step_count && blockIdx.x == 0 && threadIdx.x == 0) *p.step_ctr += 1;
   using E = typename Field<R, CPLX>::E;
   extern __shared__ __align__(128) unsigned char smem[];
   const int lane = threadIdx.x;
@@ -388,7 +388,7 @@ template <class R, bool CPLX, int AXIS, bool NORM, int L>
 __global__ void __launch_bounds__(128, CPLX ? 4 : GP_STREAM_MINB) k_sweep_stream(const SweepParams p) {
   pdl_begin();
   // the factor's dither (FP32, imaginary time): the step's x sweep has read the counter
-  if (AXIS == 1 && p.step_ctr && blockIdx.x == 0 && threadIdx.x == 0) *p.step_ctr += 1;
+  if (p.step_count && blockIdx.x == 0 && threadIdx.x == 0) *p.step_ctr += 1;
   using F = Field<R, CPLX>;
   using E = typename F::E;
   constexpr int U = kStreamU;
@@ -1624,7 +1624,7 @@ template <class R, bool CPLX, int AXIS, bool NORM, int W, bool CP>
 __global__ void __launch_bounds__(128) k_sweep_band_line(const __grid_constant__ SweepParams p) {
   pdl_begin();
   // the factor's dither (FP32, imaginary time): the step's x sweep has read the counter
-  if (AXIS == 1 && p.step_ctr && blockIdx.x == 0 && threadIdx.x == 0) *p.step_ctr += 1;
+  if (p.step_count && blockIdx.x == 0 && threadIdx.x == 0) *p.step_ctr += 1;
   using E = typename Field<R, CPLX>::E;
   LineArgs<E> a;
   a.psi = static_cast<const E*>(p.psi);

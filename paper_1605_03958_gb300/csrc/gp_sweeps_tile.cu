@@ -29,6 +29,14 @@ namespace {
 constexpr int kTileCols = 32;      // y / z: vector positions per block, one per lane
 constexpr int kTileRuns = 4;       // y / z: runs per block, one per warp
 constexpr int kBatchTileThreads = 128;   // pools: runs times columns
+constexpr int kXyThreads = 256;    // x and y together
+constexpr int kXyRows = 12;        // rows per block at most (64^3: 11.1 us a step, 15.7 with 32 rows)
+// Grids that take it (separate -> joined, us per step, real / complex): 64^3 16.1 -> 12.3 /
+// 13.3 -> 11.9, 80 x 72 x 40 12.9 -> 9.7 / 13.9 -> 10.7, 200 x 32 x 24 10.8 -> 9.7 / 12.7 -> 12.7;
+// and not: 96 x 80 x 64 12.8 -> 13.5, 256 x 32 x 32 11.5 -> 13.9 (one row a warp, 96 blocks),
+// 24 x 100 x 80 13.3 -> 14.4 (720 blocks), 8 x 160 x 160 20.8 -> 27.9 (2240)
+constexpr long long kXyPoints = 1 << 18, kXyBlocks = 400;
+constexpr int kXyWidth = 200;
 
 // points per run: one turn of the (2W+1)-point ring (W = 3: two)
 template <int W> __host__ __device__ constexpr int run_max() { return W == 3 ? 14 : 2 * W + 1; }
@@ -173,7 +181,7 @@ __global__ void __launch_bounds__(32 * kTileRuns) k_band_tile(const __grid_const
   const size_t base = (AXIS == 1 ? (size_t)o * P * p.ny : (size_t)o * P) + (on ? xv : 0);
   pdl_begin();
   // the factor's dither (FP32, imaginary time): the step's x sweep has read the counter
-  if (AXIS == 1 && p.step_ctr && blockIdx.x == 0 && threadIdx.x == 0) *p.step_ctr += 1;
+  if (p.step_count && blockIdx.x == 0 && threadIdx.x == 0) *p.step_ctr += 1;
   const float part_sum = tile_block<CPLX, NORM, W, false>(
       tile, static_cast<const float4*>(p.psi) + base, static_cast<float4*>(p.out) + base, sv, p.n, part * kTileRuns * L, L,
       kTileRuns, kTileCols, lane, run, on, min(EPT, nx - xv * EPT), p.band_wt, (long long)base, (long long)P * p.ny * p.nz,
@@ -215,6 +223,258 @@ __global__ void __launch_bounds__(kBatchTileThreads) k_batch_tile(const __grid_c
     __syncthreads();   // the tile is idle now: the norm's per-warp sums go there
     norm_finish_ff(FF{part_sum, 0.f}, reinterpret_cast<FF*>(d.partials), d.counter, (unsigned int)lb.nblk,
                    (unsigned int)lb.blk, d.scale, b.status, d.dV, nullptr, 1, reinterpret_cast<FF*>(tile));
+  }
+}
+
+// ------------------------------------------------------------------- x and y
+
+// Banded x and y sweeps in one launch, for small 3D grids: a block takes xy_rows consecutive
+// rows of one plane, plus W on each side, into shared memory, applies the pending factor, the
+// pointwise substep and the x operator to them there (a warp on its own rows, in place), and
+// then the y operator down the columns, written out of place.
+//
+// A small grid's step is a chain of latencies (launch, first loads, the norm's partials), not
+// of work, and a launch less takes a third of it away: 64 x 48 x 32 12.5 -> 8.5 us per step
+// (complex 10.9 -> 10.3), 48 x 48 x 32 12.1 -> 8.5, 33 x 60 x 50 15.5 -> 9.9 (13.2 -> 9.0).  The price is the x work of 2W halo rows a
+// block and about 78 instructions per point in all, against 35 of the separate sweeps: from
+// about 2^18 points on that is what bounds it (240 x 200 x 160: 40 us against 31; blocks of a
+// cluster that exchange their edge rows instead, 44).
+//
+// x: a lane owns eight consecutive elements of a row, 32 / lanes-per-row rows at a time; the W
+// neighbours come from the lanes beside it by shuffles, the odd images at the row's ends from
+// the lane's own and left-hand elements.  Real taps run two-lane on the pairs (e, e + 4).  Rows
+// stand in shared memory with vector v at v ^ (v >> 3 & VPL - 1), so that neither eight lanes
+// VPL vectors apart (x) nor eight neighbouring vectors (y) meet in a bank.
+// y: as in k_band_tile, one run of xy_run points per thread; the odd images of the plane's
+// first and last rows are stored along with the rows.
+template <bool CPLX, int W> struct XRow {
+  static constexpr int EPT = CPLX ? 2 : 4, VPL = 8 / EPT;
+  using F = Field<float, CPLX>;
+  using E = typename F::E;
+  E v[8], lo[W + 1], hi[W + 1];   // lo[m]: m points left of the first, hi[m]: right of the last
+  // position j of the row relative to the lane's first element
+  __device__ __forceinline__ E at(int j) const { return j < 0 ? lo[-j] : j >= 8 ? hi[j - 7] : v[j]; }
+  // images of a row that ends after the first c elements of this lane: 0 at the ghost c,
+  // -at(2c - j) at j > c
+  template <int C> __device__ __forceinline__ void end_own() {
+#pragma unroll
+    for (int j = C; j < 8; ++j) v[j] = j == C || 2 * C - j < -W ? F::zero() : F::scaled(at(2 * C - j), -1.f);
+  }
+  template <int C> __device__ __forceinline__ void end_hi() {
+#pragma unroll
+    for (int m = 1; m <= W; ++m) {
+      const int i = 2 * C - 7 - m;
+      hi[m] = i == C || i < -W ? F::zero() : F::scaled(at(i), -1.f);
+    }
+  }
+  __device__ __forceinline__ void end_own(int c) {
+    switch (c) {
+      case 1: end_own<1>(); break;
+      case 2: end_own<2>(); break;
+      case 3: end_own<3>(); break;
+      case 4: end_own<4>(); break;
+      case 5: end_own<5>(); break;
+      case 6: end_own<6>(); break;
+      case 7: end_own<7>(); break;
+    }
+  }
+  __device__ __forceinline__ void end_hi(int c) {
+    switch (c) {
+      case 1: end_hi<1>(); break;
+      case 2: end_hi<2>(); break;
+      case 3: end_hi<3>(); break;
+      case 4: end_hi<4>(); break;
+      case 5: end_hi<5>(); break;
+      case 6: end_hi<6>(); break;
+      case 7: end_hi<7>(); break;
+      default: end_hi<8>(); break;
+    }
+  }
+  // the pointwise substep by the short polynomial: the operations of
+  // Field::nonlinear_small, two real points at a time
+  __device__ __forceinline__ void small(const E (&fx)[8], E fr, float dtg) {
+    if constexpr (CPLX) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = F::nonlinear_small(v[e], F::mul(fx[e], fr), dtg * F::abs2(v[e]));
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 c = f2(v[e], v[e + 4]), z = mul2(f2(-dtg), mul2(c, c));
+        float2 q = fma2(z, f2(1.f / 24.f), f2(1.f / 6.f));
+        q = fma2(z, q, f2(0.5f));
+        q = fma2(z, q, f2(1.f));
+        q = fma2(z, q, f2(1.f));
+        const float2 r = mul2(mul2(c, mul2(f2(fx[e], fx[e + 4]), f2(fr))), q);
+        v[e] = r.x;
+        v[e + 4] = r.y;
+      }
+    }
+  }
+  __device__ __forceinline__ void start() {
+#pragma unroll
+    for (int m = 1; m <= W; ++m) lo[m] = m == 1 ? F::zero() : F::scaled(v[m - 2], -1.f);
+  }
+  __device__ __forceinline__ void result(const BandChain<CPLX, W>& taps, float4 (&o)[VPL]) const {
+    if constexpr (CPLX) {
+#pragma unroll
+      for (int q = 0; q < VPL; ++q) {
+        const float2 a = taps([&](int k) { return at(2 * q + k); });
+        const float2 b = taps([&](int k) { return at(2 * q + 1 + k); });
+        o[q] = make_float4(a.x, a.y, b.x, b.y);
+      }
+    } else {
+      float2 pr[4 + 2 * W];   // pr[W + j] = (at(j), at(j + 4))
+#pragma unroll
+      for (int j = -W; j < 4 + W; ++j) pr[W + j] = f2(at(j), at(j + 4));
+      float2 r[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) r[e] = taps([&](int k) { return pr[W + e + k]; });
+      o[0] = make_float4(r[0].x, r[1].x, r[2].x, r[3].x);
+      o[1] = make_float4(r[0].y, r[1].y, r[2].y, r[3].y);
+    }
+  }
+};
+
+template <int VPL> __device__ __forceinline__ int xy_swizzle(int v) { return v ^ ((v >> 3) & (VPL - 1)); }
+
+__device__ __forceinline__ float shfl_el(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+__device__ __forceinline__ float2 shfl_el(float2 v, int src) {
+  return f2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+
+template <bool CPLX, int W>
+__global__ void __launch_bounds__(kXyThreads) k_band_xy(const __grid_constant__ SweepParams p) {
+  extern __shared__ __align__(16) float4 tile[];
+  using F = Field<float, CPLX>;
+  using E = typename F::E;
+  using X = XRow<CPLX, W>;
+  constexpr int EPT = X::EPT, VPL = X::VPL, NW = kXyThreads / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nx = p.nx, ny = p.ny;
+  const int nl = (nx + 7) / 8, RV = nl * VPL;       // lanes of eight elements and vectors per row
+  const int RP = 32 / nl;                           // rows per warp pass
+  const int rp = lane / nl, li = lane - rp * nl;
+  const unsigned int parts = (unsigned int)p.xy_parts;
+  const int k = (int)(blockIdx.x / parts), part = (int)(blockIdx.x - (unsigned int)k * parts);
+  const int j0 = part * p.xy_rows, out_rows = min(p.xy_rows, ny - j0);
+  const int jlo = max(0, j0 - W), nreal = min(ny, j0 + out_rows + W) - jlo;
+  const int P = p.pitch / EPT;
+  const size_t plane = (size_t)k * ny * P;
+  const long long nall = (long long)P * ny * p.nz;
+  (void)nall;
+  const int npass = (nreal + RP - 1) / RP;
+  pdl_begin();
+  const float4* in = static_cast<const float4*>(p.psi) + plane;
+  for (int idx = threadIdx.x; idx < nreal * RV; idx += kXyThreads) {
+    const int row = idx / RV, v = idx - row * RV;
+    const bool ok = v < P && GP_IN((long long)plane + (long long)(jlo + row) * P + v, nall, p.status);
+    cp_async16_zfill(tile + (size_t)(jlo - j0 + W + row) * RV + xy_swizzle<VPL>(v),
+                     in + (ok ? (size_t)(jlo + row) * P + v : 0), ok);   // (past the pitch: zeros)
+  }
+  cp_async_commit();
+  // the ghost rows
+  for (int v = threadIdx.x; v < RV; v += kXyThreads) {
+    if (j0 < W) tile[(size_t)(W - 1 - j0) * RV + v] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (j0 + out_rows + W > ny) tile[(size_t)(ny - j0 + W) * RV + v] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  // the pending factor (see k_sweep_x_reg), while the rows are on their way
+  __shared__ float s_block;
+  {
+    const double f = p.norm_defer
+                         ? deferred_scale(p.partials + (size_t)(blockIdx.x % p.norm_copies) * p.norm_blocks,
+                                          p.norm_blocks, p.dV, p.status, blockIdx.x == 0, p.scale_state, p.scale)
+                         : 0.0;
+    // (rounded as the separate x sweep of such rows does)
+    const double g = p.norm_defer ? f : *p.scale;
+    if (threadIdx.x == 0)
+      s_block = p.band_reg ? (float)(g * step_dither(p.step_ctr)) : (float)g * step_dither_f(p.step_ctr);
+  }
+  const BandChain<CPLX, W> taps(p.band_wt);
+  const float dtg = p.band_dtg;
+  const bool pw = p.pw != 0;
+  const int ends = nx - 8 * (nl - 1);               // elements of a row's last lane
+  const bool first = li == 0, last = li == nl - 1;
+  const unsigned int row_lanes = nl >= 32 ? 0xffffffffu : ((1u << nl) - 1u) << (rp < RP ? rp * nl : 0);
+  E fx[8];
+#pragma unroll
+  for (int q = 0; q < VPL; ++q) {
+    const int v = li * VPL + q;
+    const float4 f = v < P ? __ldg(static_cast<const float4*>(p.band_fx) + v) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) fx[q * EPT + e] = reinterpret_cast<const E*>(&f)[e];
+  }
+  const E* fyz = static_cast<const E*>(p.band_fyz) + (size_t)k * ny + jlo;
+  cp_async_wait<0>();
+  __syncthreads();
+  const float s = s_block;
+  for (int q = warp; q < npass; q += NW) {
+    const int row = q * RP + rp;
+    const bool on = rp < RP && row < nreal;
+    const int j = jlo + row;                        // line position
+    float4* trow = tile + (size_t)(j - j0 + W) * RV;
+    const E fr = on ? fyz[row] : F::zero();
+    X x;
+    float ymax = 0.f;
+#pragma unroll
+    for (int u = 0; u < VPL; ++u) {
+      const float4 c = on ? trow[xy_swizzle<VPL>(li * VPL + u)] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int e = 0; e < EPT; ++e) x.v[u * EPT + e] = F::scaled(reinterpret_cast<const E*>(&c)[e], s);
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) ymax = fmaxf(ymax, F::abs2(x.v[e]));
+    ymax *= fabsf(dtg);   // (monotonic: the largest rounded argument)
+    // a row takes the short polynomial when every argument in it allows that
+    const unsigned int big = __ballot_sync(0xffffffffu, !(ymax <= 0.0625f));
+    if (!pw) {
+    } else if ((big & row_lanes) == 0u) {
+      x.small(fx, fr, dtg);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) x.v[e] = F::nonlinear_full(x.v[e], F::mul(fx[e], fr), dtg * F::abs2(x.v[e]));
+    }
+    // neighbours: left, the images in a ragged last lane, right
+#pragma unroll
+    for (int m = 1; m <= W; ++m) x.lo[m] = shfl_el(x.v[8 - m], (lane + 31) & 31);
+    if (first) x.start();
+    if (ends != 8 && last) x.end_own(ends);
+#pragma unroll
+    for (int m = 1; m <= W; ++m) x.hi[m] = shfl_el(x.v[m - 1], (lane + 1) & 31);
+    if (last) x.end_hi(ends);
+    float4 o[VPL];
+    x.result(taps, o);
+    if (!on) continue;
+    // the row, and its odd image about a ghost row within the block's reach
+    const int jl = -2 - j, jr = 2 * ny - j;
+    const bool il = jl >= j0 - W, ir = jr < j0 + out_rows + W;
+#pragma unroll
+    for (int u = 0; u < VPL; ++u) {
+      const int c = xy_swizzle<VPL>(li * VPL + u);
+      trow[c] = o[u];
+      if (il) tile[(size_t)(jl - j0 + W) * RV + c] = neg4(o[u]);
+      if (ir) tile[(size_t)(jr - j0 + W) * RV + c] = neg4(o[u]);
+    }
+  }
+  __syncthreads();
+  const BandTaps<CPLX, W> ytaps(p.band_wt_y);
+  const int nvec = (nx + EPT - 1) / EPT, L = p.xy_run;
+  const int items = (out_rows + L - 1) / L * nvec;
+  for (int i = threadIdx.x; i < items; i += kXyThreads) {
+    const int run = i / nvec, c = i - run * nvec, jr = run * L;
+    const size_t at = plane + (size_t)(j0 + jr) * P + c;
+    float4* out = static_cast<float4*>(p.out) + at;
+    const int valid = min(EPT, nx - c * EPT);
+    band_run<W>(tile + (size_t)jr * RV + xy_swizzle<VPL>(c), RV, min(L, out_rows - jr), ytaps, [&](int u, float4 v) {
+      if (!GP_IN((long long)at + (long long)u * P, nall, p.status)) return;
+      if (valid == EPT) {
+        *out = v;
+      } else {
+        const float e[4] = {v.x, v.y, v.z, v.w};
+        float* os = reinterpret_cast<float*>(out);
+        for (int m = 0; m < valid * (CPLX ? 2 : 1); ++m) os[m] = e[m];
+      }
+      out += P;   // (the runs emit in order)
+    });
   }
 }
 
@@ -281,6 +541,34 @@ cudaError_t launch_band_tile(int axis, const SweepParams& p, bool complex_field,
   return launch_tile(tile_kernel(axis, p.band_w, complex_field, p.plane_norm != 0), p, grid, 32 * kTileRuns,
                      tile_smem(p), st);
 }
+
+// ---- x and y
+
+static Kernel xy_kernel(int w, bool cplx) {
+  if (w == 3) return cplx ? k_band_xy<true, 3> : k_band_xy<false, 3>;
+  return cplx ? k_band_xy<true, 5> : k_band_xy<false, 5>;
+}
+
+bool band_xy_setup(SweepParams* p, bool complex_field) {
+  const int w = p->band_w;
+  const int nvec = complex_field ? (p->nx + 1) / 2 : (p->nx + 3) / 4, parts = (p->ny + kXyRows - 1) / kXyRows;
+  if ((w != 3 && w != 5) || p->nx < 8 || p->nx > kXyWidth || p->nz < 2 || (long long)p->nz * parts > kXyBlocks ||
+      (long long)p->nx * p->ny * p->nz > kXyPoints)
+    return false;
+  p->xy_rows = (p->ny + parts - 1) / parts;
+  p->xy_parts = (p->ny + p->xy_rows - 1) / p->xy_rows;
+  // at least as many runs as the threads make, of three points or more; no longer than a ring's turn
+  const int runs = std::max((p->xy_rows + run_max_of(w) - 1) / run_max_of(w), kXyThreads / nvec);
+  p->xy_run = std::max((p->xy_rows + runs - 1) / runs, std::min(p->xy_rows, 3));
+  // (at most 22 rows of 1.6 KB)
+  p->xy_smem = (p->xy_rows + 2 * w) * ((p->nx + 7) / 8) * (complex_field ? 4 : 2) * (int)sizeof(float4);
+  return true;
+}
+
+cudaError_t launch_band_xy(const SweepParams& p, bool complex_field, cudaStream_t st) {
+  return launch_tile(xy_kernel(p.band_w, complex_field), p, p.nz * p.xy_parts, kXyThreads, (size_t)p.xy_smem, st);
+}
+
 
 // ---- pools
 
