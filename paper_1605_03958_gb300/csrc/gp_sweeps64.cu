@@ -876,15 +876,21 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
           }
         } else if (live) {
           const double c2 = pw ? cy : 0.0;
+          // |y| < 2^-56: the factor alone (the far field, where |E| is large and v small: two
+          // to ten FP64 operations instead of ten to thirty; 240 x 200 x 160 at h = 0.2, where
+          // that is most of the grid: x 237 -> 119 us, complex 453 -> 264)
+          const bool quiet = !pw || vm < p.inc_quiet;
           if constexpr (!CPLX) {
             const double fr = pw ? s * static_cast<const double*>(p.band_fyz)[r0 + r] : s;
             const double* fx = static_cast<const double*>(p.band_fx);
-            v.x = pointwise64(v.x, pw ? fr * fx[2 * cv] : fr, c2);
-            v.y = pointwise64(v.y, pw ? fr * fx[2 * cv + 1] : fr, c2);
+            const double f0 = pw ? fr * fx[2 * cv] : fr, f1 = pw ? fr * fx[2 * cv + 1] : fr;
+            v.x = quiet ? v.x * f0 : pointwise64(v.x, f0, c2);
+            v.y = quiet ? v.y * f1 : pointwise64(v.y, f1, c2);
           } else {
             const double2 rf = pw ? static_cast<const double2*>(p.band_fyz)[r0 + r] : make_double2(1.0, 0.0);
             const double2 f = pw ? static_cast<const double2*>(p.band_fx)[cv] : make_double2(1.0, 0.0);
-            v = pointwise64(v, cmul(make_double2(s * f.x, s * f.y), rf), c2);
+            const double2 f0 = cmul(make_double2(s * f.x, s * f.y), rf);
+            v = quiet ? cmul(v, f0) : pointwise64(v, f0, c2);
           }
         }
       }
