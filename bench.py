@@ -209,15 +209,20 @@ def sweep_kernel_names(info, prec, real):
     c = "true" if real else "false"     # complex field
     nm = "false" if real else "true"    # the z sweep sums the norm in imaginary time only
     if info.get("line64_mask", 0) == 7:
-        return {"sweep_x": f"k_sweep_x64<{c}>", "sweep_y": f"k_sweep_line64<{c},1,false>",
-                "sweep_z": f"k_sweep_line64<{c},2,{nm}>"}
+        inc = info["inc64_mask"]
+        return {"sweep_x": f"k_sweep_xinc64<{c}>" if inc & 1 else f"k_sweep_x64<{c}>",
+                "sweep_y": f"k_sweep_inc64<{c},1,false>" if inc & 2 else f"k_sweep_line64<{c},1,false>",
+                "sweep_z": f"k_sweep_inc64<{c},2,{nm}>" if inc & 4 else f"k_sweep_line64<{c},2,{nm}>"}
+    tile = info["tile_mask"]
     return {
         "sweep_x": (f"k_sweep_x_reg<{c},{W}>" if info.get("x_reg") else
                     f"k_sweep_x_band<float,{c},{W}>" if info["band_mask"] & 1 else
                     f"k_sweep_x_stream<float,{c},{L}>" if info["fast_mask"] & 1 else f"k_sweep_x<{rt},{c}>"),
-        "sweep_y": (f"k_sweep_band_line<float,{c},1,false,{W}>" if info["band_mask"] & 2 else
+        "sweep_y": (f"k_band_tile<{c},1,false,{W}>" if tile & 2 else
+                    f"k_sweep_band_line<float,{c},1,false,{W}>" if info["band_mask"] & 2 else
                     f"k_sweep_stream<float,{c},1,false,{L}>" if info["fast_mask"] & 2 else f"k_sweep_y<{rt},{c}>"),
-        "sweep_z": (f"k_sweep_band_line<float,{c},2,{nm},{W}>" if info["band_mask"] & 4 else
+        "sweep_z": (f"k_band_tile<{c},2,{nm},{W}>" if tile & 4 else
+                    f"k_sweep_band_line<float,{c},2,{nm},{W}>" if info["band_mask"] & 4 else
                     f"k_sweep_stream<float,{c},2,{nm},{L}>" if info["fast_mask"] & 4 else f"k_sweep_z<{rt},{c},{nm}>")}
 
 
@@ -271,6 +276,10 @@ def time_steps(P, so, step, steps, flush):
 # + forward (4 / 14) + back substitution (1 / 4); y and z: 5 / 18; the imaginary-time
 # z sweep adds 1 for the norm.
 FP64_OPS = {"imag": (13, 5, 6), "real": (39, 18, 18)}
+# In increment form (k_sweep_xinc64, k_sweep_inc64) one addition per value and sweep is left,
+# in x another for the substep, and the norm's in z; the rest is two-part FP32, whose issue is
+# what bounds those sweeps.
+FP64_OPS_INC = {"imag": (2, 1, 2), "real": (4, 2, 2)}
 
 
 def fp64_peak():
@@ -319,8 +328,8 @@ def paper_precision(P, args, flush, hbm, sm_mhz):
         so, st = make_workload_solver(P, "f64", mode, grid)
         ms, sw, kn = time_steps(P, so, st, steps, flush)
         names = sweep_kernel_names(so.info(), "f64", mode == "real")
+        ops = (FP64_OPS_INC if so.info()["inc64_mask"] == 7 else FP64_OPS)[mode]
         so.close()
-        ops = FP64_OPS[mode]
         sb = 16 if mode == "real" else 8
         per = {}
         for i, n in enumerate(("sweep_x", "sweep_y", "sweep_z")):
@@ -623,7 +632,7 @@ def run_cuda(args):
         # dominant sweep against the FP64 ALU peak (the HBM figures stay in `sweeps`)
         sm_mhz = (clk.summary() or {}).get("sm_mhz") or 2070.0
         fpk, nsm = fp64_pipe_peak(sm_mhz)
-        ops = FP64_OPS["real" if real else "imag"][names.index(dom)]
+        ops = (FP64_OPS_INC if info["inc64_mask"] == 7 else FP64_OPS)["real" if real else "imag"][names.index(dom)]
         ach = ops * NPTS / (per[dom]["avg_ms"] / 1e3)
         roofline = {"bound": "alu", "kernel": kernels[dom], "achieved": round(ach / 1e12, 4),
                     "peak": round(fpk / 1e12, 4), "unit": "T FP64 op/s",

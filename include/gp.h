@@ -259,7 +259,10 @@ int gp_get_timing(gp_solver* s, double ms[3], long long launches[3]);
  *           gp_sweeps.cu), bit 3 + a when that kernel is the banded operator, bits
  *           8..11 the largest band half-width W, bits 12 + a when sweep a uses the
  *           FP64 line-streaming kernels (FP64 field; gp_sweeps64.cu), bit 15 when the
- *           banded x sweep holds each row in registers (k_sweep_x_reg),
+ *           banded x sweep holds each row in registers (k_sweep_x_reg), bits 16 + a when
+ *           banded sweep a goes over shared-memory tiles (k_band_tile), bits 19 + a when
+ *           FP64 sweep a takes the increment form, bit 22 when the x and y sweeps are one
+ *           launch (k_band_xy),
  *   info[7] the truncation depth L of the streaming recurrences (0 when none).
  * GP_SWEEP_KERNELS=tile in the environment at gp_create time makes every sweep
  * use the tile kernels; =stream keeps the FP32 sweeps on the streaming recurrences

@@ -973,8 +973,11 @@ struct NvtxRange {
   ~NvtxRange() { nvtxRangePop(); }
 };
 
-// x and y in one pass: wherever set up, except while sweeps are timed one by one.
-bool xy_joined(const gp_solver* s) { return s->sp_xy[s->is_complex ? 1 : 0].xy_parts > 0 && !s->timing; }
+// x and y in one pass: wherever set up, except while sweeps are timed one by one or a wait
+// limit other than the default asks for the copy-fed x sweep's bounded waits.
+bool xy_joined(const gp_solver* s) {
+  return s->sp_xy[s->is_complex ? 1 : 0].xy_parts > 0 && !s->timing && s->sp[0][0].wait_ns == gpk::kWaitLimitNs;
+}
 
 int run_xy(gp_solver* s) {
   NvtxRange range("gp sweep xy");
@@ -1689,6 +1692,11 @@ int gp_get_info(const gp_solver* s, long long info[8]) {
   info[6] |= (long long)wmax << 8;
   if (s->line64) info[6] |= 7LL << 12;
   if (s->sp[m][0].band_reg) info[6] |= 1LL << 15;
+  for (int a = 0; a < 3; ++a) {
+    if (a > 0 && s->band_w[m][a] && s->sp[m][a].band_cp == 2) info[6] |= 1LL << (16 + a);
+    if (s->line64 && s->sp[m][a].inc_x) info[6] |= 1LL << (19 + a);
+  }
+  if (s->sp_xy[m].xy_parts) info[6] |= 1LL << 22;
   info[7] = std::max(s->trunc[m][0], std::max(s->trunc[m][1], s->trunc[m][2]));
   return GP_OK;
 }

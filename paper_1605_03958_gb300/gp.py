@@ -312,6 +312,9 @@ def gp_get_info(h) -> dict:
     d["band_w"] = (d["fast_mask"] >> 8) & 15
     d["line64_mask"] = (d["fast_mask"] >> 12) & 7
     d["x_reg"] = (d["fast_mask"] >> 15) & 1
+    d["tile_mask"] = (d["fast_mask"] >> 16) & 7
+    d["inc64_mask"] = (d["fast_mask"] >> 19) & 7
+    d["xy"] = (d["fast_mask"] >> 22) & 1
     d["fast_mask"] &= 7
     return d
 
