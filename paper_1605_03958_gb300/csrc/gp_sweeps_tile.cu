@@ -30,13 +30,13 @@ constexpr int kTileCols = 32;      // y / z: vector positions per block, one per
 constexpr int kTileRuns = 4;       // y / z: runs per block, one per warp
 constexpr int kBatchTileThreads = 128;   // pools: runs times columns
 constexpr int kXyThreads = 256;    // x and y together
-constexpr int kXyRows = 12;        // rows per block at most (64^3: 11.1 us a step, 15.7 with 32 rows)
-// Grids that take it (separate -> joined, us per step, real / complex): 64^3 16.1 -> 12.3 /
-// 13.3 -> 11.9, 80 x 72 x 40 12.9 -> 9.7 / 13.9 -> 10.7, 200 x 32 x 24 10.8 -> 9.7 / 12.7 -> 12.7;
-// and not: 96 x 80 x 64 12.8 -> 13.5, 256 x 32 x 32 11.5 -> 13.9 (one row a warp, 96 blocks),
-// 24 x 100 x 80 13.3 -> 14.4 (720 blocks), 8 x 160 x 160 20.8 -> 27.9 (2240)
-constexpr long long kXyPoints = 1 << 18, kXyBlocks = 400;
-constexpr int kXyWidth = 200;
+constexpr int kXyRows = 12;        // rows per block at most (64^3: 11.1 us a step, 15.7 with 32)
+// Grids that take it (separate -> joined, us per step, real / complex): 64^3 11.1 -> 9.2 /
+// 10.4 -> 8.9, 96 x 80 x 64 11.7 -> 10.7 / 12.1 -> 11.1, 256 x 32 x 32 10.1 -> 9.6 / 10.3 -> 9.5;
+// and not: 131 x 97 x 61 15.4 -> 18.3 / 15.9 -> 20.0, 24 x 100 x 80 (720 blocks) 12.8 -> 13.3 /
+// 12.1 -> 11.5
+constexpr long long kXyPoints = 1 << 19, kXyBlocks = 600;
+constexpr int kXyWidth = 256;      // a warp's lanes
 
 // points per run: one turn of the (2W+1)-point ring (W = 3: two)
 template <int W> __host__ __device__ constexpr int run_max() { return W == 3 ? 14 : 2 * W + 1; }
@@ -234,10 +234,10 @@ __global__ void __launch_bounds__(kBatchTileThreads) k_batch_tile(const __grid_c
 // then the y operator down the columns, written out of place.
 //
 // A small grid's step is a chain of latencies (launch, first loads, the norm's partials), not
-// of work, and a launch less takes a third of it away: 64 x 48 x 32 12.5 -> 8.5 us per step
-// (complex 10.9 -> 10.3), 48 x 48 x 32 12.1 -> 8.5, 33 x 60 x 50 15.5 -> 9.9 (13.2 -> 9.0).  The price is the x work of 2W halo rows a
+// of work, and a launch less takes a third of it away: 64 x 48 x 32 9.8 -> 8.3 us per step
+// (complex 9.3 -> 7.5), 33 x 60 x 50 12.1 -> 8.7 (10.8 -> 8.7).  The price is the x work of 2W halo rows a
 // block and about 78 instructions per point in all, against 35 of the separate sweeps: from
-// about 2^18 points on that is what bounds it (240 x 200 x 160: 40 us against 31; blocks of a
+// about 2^19 points on that is what bounds it (240 x 200 x 160: 40 us against 31; blocks of a
 // cluster that exchange their edge rows instead, 44).
 //
 // x: a lane owns eight consecutive elements of a row, 32 / lanes-per-row rows at a time; the W
@@ -560,7 +560,7 @@ bool band_xy_setup(SweepParams* p, bool complex_field) {
   // at least as many runs as the threads make, of three points or more; no longer than a ring's turn
   const int runs = std::max((p->xy_rows + run_max_of(w) - 1) / run_max_of(w), kXyThreads / nvec);
   p->xy_run = std::max((p->xy_rows + runs - 1) / runs, std::min(p->xy_rows, 3));
-  // (at most 22 rows of 1.6 KB)
+  // (at most 22 rows of 2 KB)
   p->xy_smem = (p->xy_rows + 2 * w) * ((p->nx + 7) / 8) * (complex_field ? 4 : 2) * (int)sizeof(float4);
   return true;
 }

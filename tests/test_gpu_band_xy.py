@@ -1,6 +1,6 @@
 """Banded x and y sweeps in one launch (k_band_xy, small 3D FP32 grids) against the two
 separate sweeps: the same operations in the same order, so the same bits, as long as a row
-takes the short polynomial in both.  Rows of one lane and of 25, ragged ends of every
+takes the short polynomial in both.  Rows of one lane and of all 32, ragged ends of every
 length, blocks of one row and of twelve, planes with a single block (both images in reach),
 half-widths 3 and 5, a row too wide for it, both modes and splittings, steps by the graph and by direct launches.
 """
@@ -22,7 +22,8 @@ def P():
 
 
 SHAPES = [(8, 8, 8), (9, 13, 8), (15, 12, 9), (33, 25, 10), (37, 11, 8), (64, 48, 32), (100, 8, 20),
-          (197, 37, 8), (199, 24, 9), (200, 32, 32), (201, 24, 8), (8, 8, 200)]
+          (197, 37, 8), (199, 24, 9), (200, 32, 32), (255, 24, 9), (256, 32, 32),
+          (257, 24, 8), (8, 8, 200)]
 
 
 @pytest.mark.parametrize("shape", SHAPES + [(16 + r, 14, 8) for r in range(8)])
