@@ -1089,7 +1089,7 @@ cudaError_t launch_inc64(int axis, const SweepParams& p, bool complex_field, cud
   cfg.dynamicSmemBytes = (size_t)(kIncL + 2) * cfg.blockDim.x * sizeof(float4);
   if (axis == 0) {
     // grids of at most two blocks per SM: more threads than segments share the passes along
-    // the rows (64 x 48 x 32: x 22.5 -> 19.3 us, 101 x 77 x 53 complex step 75 -> 58 us; larger
+    // the rows (64 x 48 x 32, then 24 blocks: x 22.5 -> 19.3 us, 101 x 77 x 53 complex step 75 -> 58 us; larger
     // grids would lose resident blocks)
     if (cfg.gridDim.x <= 304) cfg.blockDim.x = kIncThreads;
     cfg.dynamicSmemBytes = inc64_x_smem(cfg.blockDim.x, p.inc_x);

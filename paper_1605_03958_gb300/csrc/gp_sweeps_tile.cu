@@ -13,7 +13,8 @@
 // once, and the taps are two-lane FP32 (6.5 FP32 instructions per point instead of 12).
 // Measured per step (GB300; k_sweep_band_line -> here): 131 x 97 x 61 real 21.1 -> 16.9 us,
 // complex 21.3 -> 19.2; 300 x 256 plane 10.6 -> 8.2, complex 9.2 -> 7.4; 64 x 48 x 32 13.7 ->
-// 11.9; 240 x 200 x 160 31.9 -> 30.6, complex 66.6 -> 64.4.  What bounds it at 240 x 200 x 160:
+// 11.9; 240 x 200 x 160 31.9 -> 30.6, complex 66.6 -> 64.4 (since the next sweep's blocks are let
+// in at exit 131 x 97 x 61 takes 15.2 and 15.8, the plane 8.0, 240 x 200 x 160 complex 61.3).  What bounds it at 240 x 200 x 160:
 // issue and latency together (2.3 instructions per clock, 22 warps per SM); a copy of the
 // field takes 8.3 us where a sweep takes 14.
 #include <algorithm>
