@@ -405,6 +405,9 @@ void resolve_scale(gp_solver* s) {
   if (e != cudaSuccess) cuda_fail(s, e, "resolve scale");
 }
 
+// The words of an FP64 field's largest value (kAmax*), behind the step count.
+int* amax_words(const gp_solver* s) { return reinterpret_cast<int*>(s->step_ctr) + 1; }
+
 // Arguments of the reductions, I/O and pointwise kernels, which all read the pending
 // factor: a deferred one is resolved first.
 FieldParams field_params(gp_solver* s) {
@@ -425,6 +428,7 @@ FieldParams field_params(gp_solver* s) {
   f.hy = s->prm.dy;
   f.hz = s->prm.nz == 1 ? 1.0 : s->prm.dz;   // 2D: cell area hx hy
   f.g = s->g;
+  f.amax = s->line64 ? amax_words(s) : nullptr;
   return f;
 }
 
@@ -506,7 +510,7 @@ void fill_sweep_params(gp_solver* s) {
         // the increment form where the line qualifies (one norm partial per block)
         const double h = a == 0 ? p.dx : a == 1 ? p.dy : p.dz, beta = p.dt / (4.0 * h * h);
         q.inc_ex = coef + s->L.ex_off[m];
-        q.inc_amax = reinterpret_cast<int*>(s->step_ctr) + 1;
+        q.inc_amax = amax_words(s);
         if (!gpk::inc64_setup(a, &q, m == 0 ? std::complex<double>(beta, 0.0)
                                              : std::complex<double>(0.0, beta), m == 1) ||
             (a > 0 && gpk::inc64_blocks(a, q, m == 1) > (long long)s->L.npartials))
@@ -840,11 +844,10 @@ int set_scale_one(gp_solver* s) {
 }
 
 // A new field: its imaginary-time steps (the FP32 factor's dither) count from zero, and
-// nothing is known of its largest value (the two words behind the count: the FP64
-// increment sweeps' noise floor), so that the same field and the same steps give the same
-// bits in any solver.
+// nothing is known of its largest value until its kernel has written it (FP64: call this
+// first), so that the same field and the same steps give the same bits in any solver.
 int reset_steps(gp_solver* s) {
-  GP_CUDA(s, cudaMemsetAsync(s->step_ctr, 0, 3 * sizeof(unsigned int), s->stream));
+  GP_CUDA(s, cudaMemsetAsync(s->step_ctr, 0, (1 + gpk::kAmaxWords) * sizeof(unsigned int), s->stream));
   return GP_OK;
 }
 
@@ -1249,6 +1252,7 @@ int promote_to_complex(gp_solver* s) {
   if (e != cudaSuccess) return cuda_fail(s, e, "export");
   s->is_complex = true;
   f = field_params(s);
+  GP_CUDA(s, cudaMemsetAsync(amax_words(s), 0, gpk::kAmaxWords * sizeof(int), s->stream));
   e = is_f64(s) ? gpk::launch_import<double>(f, s->staging, true, s->stream)
                 : gpk::launch_import<float>(f, s->staging, true, s->stream);
   if (e != cudaSuccess) return cuda_fail(s, e, "import");
@@ -1352,6 +1356,7 @@ int gp_init_gaussian(gp_solver* s, double wx, double wy, double wz) {
       !std::isfinite(wz))
     return fail(s, GP_ERR_ARG, "Gaussian frequencies must be finite and > 0");
   s->is_complex = false;
+  if (const int rc_ = reset_steps(s)) return rc_;
   FieldParams f = field_params(s);
   f.out = s->scale;
   cudaError_t e = is_f64(s) ? gpk::launch_init_gaussian<double>(f, wx, wy, wz, s->stream)
@@ -1359,8 +1364,7 @@ int gp_init_gaussian(gp_solver* s, double wx, double wy, double wz) {
   if (e != cudaSuccess) return cuda_fail(s, e, "init_gaussian");
   e = is_f64(s) ? gpk::launch_norm_to_scale<double>(f, s->stream)
                 : gpk::launch_norm_to_scale<float>(f, s->stream);
-  if (e != cudaSuccess) return cuda_fail(s, e, "norm");
-  return reset_steps(s);
+  return e == cudaSuccess ? GP_OK : cuda_fail(s, e, "norm");
 }
 
 int gp_set_psi(gp_solver* s, const double* host, int is_complex) {
@@ -1370,12 +1374,12 @@ int gp_set_psi(gp_solver* s, const double* host, int is_complex) {
   GP_CUDA(s, cudaMemcpyAsync(s->staging, host, N * 8 * (is_complex ? 2 : 1),
                              cudaMemcpyHostToDevice, s->stream));
   s->is_complex = is_complex == 1;
+  if (const int rc_ = reset_steps(s)) return rc_;
   const FieldParams f = field_params(s);
   cudaError_t e = is_f64(s) ? gpk::launch_import<double>(f, s->staging, s->is_complex, s->stream)
                             : gpk::launch_import<float>(f, s->staging, s->is_complex, s->stream);
   if (e != cudaSuccess) return cuda_fail(s, e, "import");
-  const int rc = set_scale_one(s);
-  return rc != GP_OK ? rc : reset_steps(s);
+  return set_scale_one(s);
 }
 
 int gp_get_psi(gp_solver* s, double* host, int as_complex) {

@@ -157,6 +157,10 @@ template <int N> __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// The high word of |v|, ordered as |v| is (complex: of the larger component).
+__device__ __forceinline__ int high_word(double v) { return __double2hiint(v) & 0x7fffffff; }
+__device__ __forceinline__ int high_word(double2 v) { return max(high_word(v.x), high_word(v.y)); }
+
 // Programmatic dependent launch: wait until the previous kernel has completed and its memory
 // operations are visible (a no-op for a kernel launched without the programmatic-
 // serialization attribute).  The next kernel's blocks are let in as this kernel's blocks exit,

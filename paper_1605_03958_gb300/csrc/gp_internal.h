@@ -106,7 +106,7 @@ struct SweepParams {
   double rho[2];
   float rho_f[4];
   int inc_quiet;         // x: high word of |v| below which the nonlinear term is nothing
-  int* inc_amax;         // the field's largest |v| as an FP64 high word (see inc_floor)
+  int* inc_amax;         // FP64: words of the field's largest value (kAmax*)
   const void* inc_ex;    // x: trap factor along x less 1, two-part FP32, per 16-byte vector of a row:
                          // (h, h', l, l') of two real columns or of (re, im) of one complex
   // pointwise substep (x sweep only)
@@ -186,6 +186,17 @@ struct BatchArgs {
   int x_reg;              // x: rows in registers (k_batch_x_reg), items of `group` rows per pass
 };
 
+// FP64 solves: the largest component of the field, as the high word of an FP64 number, in
+// kAmaxWords integers.  Words are written by one launch and read by later ones only, so that
+// no block order shows, and none outlives its step:
+//   kAmaxNow   the field as set (import, Gaussian), then as the latest finished x sweep left
+//              it: read by x and z
+//   kAmaxStep  steps counted by y; x copies it to kAmaxCopy for y, which must not read what
+//              it counts
+//   kAmaxMax   two maxima by the parity of the step: x adds to one; y reads it, moves it to
+//              kAmaxNow and clears the other for the next step
+constexpr int kAmaxNow = 0, kAmaxStep = 1, kAmaxCopy = 2, kAmaxMax = 3, kAmaxWords = 5;
+
 // Arguments of the reductions and conversion kernels.
 struct FieldParams {
   void* psi;
@@ -197,6 +208,7 @@ struct FieldParams {
   int* status;
   const double* tab;     // FP64 tables: V_x[nx] V_y[ny] V_z[nz] x^2[nx] y^2[ny] z^2[nz]
   double hx, hy, hz, g;
+  int* amax = nullptr;   // FP64 solves: kAmaxNow receives the values written (import, Gaussian); else null
 };
 
 // Kernel launchers (gp_sweeps.cu / gp_reduce.cu).  R = double or float storage.

@@ -478,10 +478,19 @@ __global__ void k_import_f32(const FieldParams p, int words, const float* __rest
 
 // ------------------------------------------------------------ initial Gaussian
 
+// The largest of the values a block's threads wrote (vmax: their high words) into the field's
+// word; every thread of the block calls it.
+__device__ __forceinline__ void field_max(int vmax, int* amax) {
+  if (!amax) return;
+  vmax = __reduce_max_sync(0xffffffffu, vmax);
+  if ((threadIdx.x & 31) == 0) atomicMax(amax + kAmaxNow, vmax);
+}
+
 template <class R>
 __global__ void k_init_gaussian(const FieldParams p, double wx, double wy, double wz) {
   const int nx = p.nx, ny = p.ny, P = p.pitch;
   const long long nrows = (long long)ny * p.nz;
+  int vmax = 0;
   for (long long r = blockIdx.x; r < nrows; r += gridDim.x) {
     const int j = (int)(r % ny), k = (int)(r / ny);
     const double y = (j - 0.5 * (ny - 1)) * p.hy;
@@ -493,8 +502,10 @@ __global__ void k_init_gaussian(const FieldParams p, double wx, double wy, doubl
         v = exp(-0.5 * (wx * x * x + wy * y * y + wz * z * z));
       }
       static_cast<R*>(p.psi)[(size_t)r * P + i] = (R)v;
+      vmax = max(vmax, high_word(v));
     }
   }
+  field_max(vmax, p.amax);
 }
 
 // ------------------------------------------------- host layout <-> device field
@@ -504,17 +515,20 @@ __global__ void k_import(const FieldParams p, const double* __restrict__ src) {
   using C = typename Cplx<R>::T;
   const int nx = p.nx, P = p.pitch;
   const long long nrows = (long long)p.ny * p.nz;
+  int vmax = 0;
   for (long long r = blockIdx.x; r < nrows; r += gridDim.x)
     for (int i = threadIdx.x; i < P; i += blockDim.x) {
       const size_t d = (size_t)r * P + i, q = (size_t)r * nx + i;
+      const double re = i >= nx ? 0.0 : CPLX ? src[2 * q] : src[q];
+      const double im = CPLX && i < nx ? src[2 * q + 1] : 0.0;
+      vmax = max(vmax, max(high_word(re), high_word(im)));
       if (CPLX) {
-        C v{R(0), R(0)};
-        if (i < nx) v = C{(R)src[2 * q], (R)src[2 * q + 1]};
-        static_cast<C*>(p.psi)[d] = v;
+        static_cast<C*>(p.psi)[d] = C{(R)re, (R)im};
       } else {
-        static_cast<R*>(p.psi)[d] = i < nx ? (R)src[q] : R(0);
+        static_cast<R*>(p.psi)[d] = (R)re;
       }
     }
+  field_max(vmax, p.amax);
 }
 
 template <class R, bool CPLX>

@@ -177,6 +177,23 @@ template <bool CPLX> struct X64Geom {
   static constexpr size_t smem = kX64Warps * warp_elems * sizeof(E);
 };
 
+// x: the parity of the step whose maximum it adds to (one thread of the launch also leaves
+// the step count for y); y: that maximum, and the end of the step (one thread of the launch).
+__device__ __forceinline__ int amax_parity(int* amax, bool one) {
+  const int n = amax[kAmaxStep];
+  if (one) amax[kAmaxCopy] = n;
+  return n & 1;
+}
+__device__ __forceinline__ int amax_of_step(const int* amax) {
+  return amax[kAmaxMax + (amax[kAmaxCopy] & 1)];
+}
+__device__ __forceinline__ void amax_end_step(int* amax) {
+  const int n = amax[kAmaxCopy];
+  amax[kAmaxNow] = amax[kAmaxMax + (n & 1)];
+  amax[kAmaxMax + (~n & 1)] = 0;
+  amax[kAmaxStep] = (int)((unsigned int)n + 1u);
+}
+
 template <bool CPLX>
 __global__ void __launch_bounds__(kX64Warps * 32) k_sweep_x64(const __grid_constant__ SweepParams p) {
   using F = Field<double, CPLX>;
@@ -191,7 +208,9 @@ __global__ void __launch_bounds__(kX64Warps * 32) k_sweep_x64(const __grid_const
   const long long nrows = (long long)p.ny * p.nz;
   const long long r0 = ((long long)blockIdx.x * kX64Warps + wib) * 32;
   pdl_begin();
+  const int par = amax_parity(p.inc_amax, blockIdx.x == 0 && threadIdx.x == 0);
   if (r0 >= nrows) return;
+  int vmax = 0;
   const int rows = (int)min(32LL, nrows - r0);
   const int nx = p.nx, P = p.pitch, head = p.head;
   E* field = static_cast<E*>(p.psi) + (size_t)r0 * P;
@@ -242,7 +261,10 @@ __global__ void __launch_bounds__(kX64Warps * 32) k_sweep_x64(const __grid_const
         pointwise_cplx<NG>(xv, rf, Gc, cy);
       }
 #pragma unroll
-      for (int u = 0; u < NG; ++u) b[(g0 + u * RPI + lr) * LD + lc] = xv[u];
+      for (int u = 0; u < NG; ++u) {
+        vmax = imax(vmax, high_word(xv[u]));
+        b[(g0 + u * RPI + lr) * LD + lc] = xv[u];
+      }
     }
   };
   // chunk c of b to the field, lane = column
@@ -300,6 +322,8 @@ __global__ void __launch_bounds__(kX64Warps * 32) k_sweep_x64(const __grid_const
     // the last chunk's forward values stay in shared memory for the back substitution
     if (c + 1 < nch) store_chunk(c, buf(c));
   }
+  vmax = __reduce_max_sync(0xffffffffu, vmax);
+  if (lane == 0) atomicMax(p.inc_amax + kAmaxMax + par, vmax);
   for (int c = nch - 1; c >= 0; --c) {
     E* b = buf(c);
     if (c + 1 < nch) {
@@ -328,6 +352,7 @@ __global__ void __launch_bounds__(kLineThreads) k_sweep_line64(const __grid_cons
   using F = Field<double, CPLX>;
   using E = typename F::E;
   pdl_begin();
+  if (AXIS == 1 && blockIdx.x == 0 && threadIdx.x == 0) amax_end_step(p.inc_amax);
   const int nx = p.nx, n = p.n, head = p.head;
   const long long nlines = (long long)nx * (AXIS == 1 ? p.nz : p.ny);
   const long long g = (long long)blockIdx.x * kLineThreads + threadIdx.x;
@@ -436,12 +461,9 @@ constexpr int kIncThreads = 256; // most threads per block
 constexpr int kIncSms = 152;     // SMs of a GB300
 
 // Noise is looked for in values above 2^-10 of the field's largest (noise below that, in
-// the far tails, adds nothing to the field's error).  The x sweep takes the largest FP64 high
-// word (as an integer, so the order of the blocks does not matter) into amax[0]; the y
-// sweep uses it and copies it to amax[1], which the z sweep and the next x sweep use; the
-// z sweep clears amax[0].  Zero (a new field, no x sweep of this form): no floor.
-__device__ __forceinline__ float inc_floor(const int* amax) {
-  const int t = addmax0(*amax, -kSplitOff);
+// the far tails, adds nothing to the field's error); amax: its high word.
+__device__ __forceinline__ float inc_floor(int amax) {
+  const int t = addmax0(amax, -kSplitOff);
   return t >= kSplitTooBig ? 0.f : bits_f((uint32_t)t << 3) * 0x1p-10f;
 }
 
@@ -667,11 +689,8 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_inc64(const __grid_consta
   cp_async_commit();
   const double2 before = io.rd(j0 - 1), after = io.rd(j0 + kIncL);
   const IncRho<CPLX> rho(p);
-  const float least = inc_floor(p.inc_amax + (AXIS == 1 ? 0 : 1));
-  if (blockIdx.x == 0 && tid == 0) {
-    if (AXIS == 1) p.inc_amax[1] = p.inc_amax[0];
-    else p.inc_amax[0] = 0;
-  }
+  const float least = inc_floor(AXIS == 1 ? amax_of_step(p.inc_amax) : p.inc_amax[kAmaxNow]);
+  if (AXIS == 1 && blockIdx.x == 0 && tid == 0) amax_end_step(p.inc_amax);
   cp_async_wait<0>();
   inc_segment<CPLX>(rho, slot, T, carry, T, X, sg, nseg, j0, n, io.on, before, after, least, io);
   if constexpr (NORM) norm_finish(io.acc, p.partials, p.counter, gridDim.x, blockIdx.x, p.scale_out,
@@ -749,7 +768,7 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
   (void)nall;
   (void)at0;
   __shared__ double head_d[3];   // the factor applied ahead, the one folded in, dt g s^2
-  __shared__ int head_max;
+  __shared__ int head_max, head_now;   // the block's largest value, the field's before the substep
   const IncRho<CPLX> rho(p);
   pdl_begin();
   // FP64 is slow even a few operations per thread: one thread forms the block's scalars
@@ -761,9 +780,13 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
     head_d[1] = fold ? s : 1.0;
     head_d[2] = p.dt * p.g * head_d[1] * head_d[1];
     head_max = 0;
+    // (kAmaxNow is that of the field without its pending factor)
+    const int now = p.inc_amax[kAmaxNow];
+    head_now = fold ? now : high_word(__hiloint2double(now, 0) * s);
   }
-  const float least = inc_floor(p.inc_amax + 1);
+  const int par = amax_parity(p.inc_amax, blockIdx.x == 0 && tid == 0);
   __syncthreads();
+  const float least = inc_floor(head_now);
   const double spre = head_d[0], s = head_d[1], cy = head_d[2];
   const bool pre = __double2hiint(spre) != 0x3ff00000 || __double2loint(spre) != 0;
   const bool pw = p.pw != 0;
@@ -824,7 +847,7 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
         v.x *= spre;
         v.y *= spre;
       }
-      const int vm = imax(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff);
+      const int vm = high_word(v);
       vmax = imax(vmax, vm);
       if (work) {
         const float4* rc = rowc + (CPLX ? 3 : 1) * (live ? r : 0);
@@ -910,7 +933,7 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
   vmax = __reduce_max_sync(0xffffffffu, vmax);
   if ((tid & 31) == 0) atomicMax(&head_max, vmax);
   __syncthreads();
-  if (tid == 0) atomicMax(p.inc_amax, head_max);
+  if (tid == 0) atomicMax(p.inc_amax + kAmaxMax + par, head_max);
   {
     const int sg = tid / X, xl = tid - sg * X;
     const int j0 = sg * kIncL;

@@ -1,0 +1,82 @@
+"""FP64 steps against the same steps in extended precision (numpy's long double): fields on
+which arithmetic in two FP32 parts has no bits to spare.
+
+Tolerance: a step is four substeps, and whichever way a substep is evaluated its relative L2
+error is to stay within 2^-53, that of the FP64 operations it replaces (an FP64 recurrence or
+product of factors measures 0.9e-16..1.2e-16); the substeps' roundings are independent:
+sqrt(4 steps) 2^-53."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+W = (1.0, 1.41, 2.0)
+
+
+@pytest.fixture(scope="module")
+def P():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1605_03958_gb300 as pkg
+    return pkg
+
+
+def solve(u, axis, a):
+    """(I + aK)^-1 (I - aK) u along an axis, K the second difference with zero ghosts."""
+    u = np.moveaxis(u, axis, 0)
+    n = u.shape[0]
+    r = (1 - 2 * a) * u
+    r[1:] += a * u[:-1]
+    r[:-1] += a * u[1:]
+    c = np.empty(n, u.dtype)
+    for j in range(n):
+        den = 1 + 2 * a + (a * c[j - 1] if j else 0)
+        c[j] = -a / den
+        r[j] = (r[j] + (a * r[j - 1] if j else 0)) / den
+    for j in range(n - 2, -1, -1):
+        r[j] -= c[j] * r[j + 1]
+    return np.moveaxis(r, 0, axis)
+
+
+def exact(shape, h, dt, g, mode, psi, steps):
+    Q = np.longdouble
+    u = psi.astype(np.clongdouble if mode == "real" else Q)
+    x, y, z = ((np.arange(n) - Q(0.5) * (n - 1)) * Q(h) for n in shape)
+    V = sum(Q(w) ** 2 / 2 * q * q for w, q in zip(W, (x[None, None, :], y[None, :, None], z[:, None, None])))
+    a = Q(dt) / (4 * Q(h) * Q(h)) * (1j if mode == "real" else 1)
+    axes = (2, 1) if shape[2] == 1 else (2, 1, 0)
+    for _ in range(steps):
+        d = Q(dt) * (V + Q(g) * (u.real * u.real + (u.imag * u.imag if mode == "real" else 0)))
+        u = u * (np.cos(d) - 1j * np.sin(d) if mode == "real" else np.exp(-d))
+        for ax in axes:
+            u = solve(u, ax, a)
+        if mode == "imag":
+            u = u / np.sqrt((u * u).sum() * Q(h) ** len(axes))
+    return u
+
+
+def check(P, shape, h, dt, g, mode, psi, steps):
+    s = P.Solver(*shape, h, dt=dt, gamma=W[0], nu=W[1], lam=W[2], g=g, prec="f64")
+    s.set_psi(psi)
+    (s.step_real if mode == "real" else s.step_imag)(steps)
+    got = s.get_psi(as_complex=mode == "real")
+    s.close()
+    ref = exact(shape, h, dt, g, mode, psi, steps)
+    err = float(np.sqrt((abs(got - ref) ** 2).sum() / (abs(ref) ** 2).sum()))
+    assert err <= np.sqrt(4 * steps) * 2.0 ** -53, err
+
+
+def noise(shape, mode, seed=3):
+    rng = np.random.default_rng(seed)
+    f = 0.3 * rng.standard_normal(shape[::-1])
+    return f + 0.3j * rng.standard_normal(f.shape) if mode == "real" else f
+
+
+@pytest.mark.parametrize("shape", [(512, 304, 1), (512, 64, 9)])
+def test_noise_in_a_field_that_has_fallen(P, shape):
+    """Grids without an increment sweep along z (planes, nz < 16), noise 2^20 above its
+    normalised size at the start: what counts as noise follows the field down."""
+    h = 0.05   # (a trap whose factor stays near 1 over the whole grid)
+    check(P, shape, h, 0.1 * h * h, 0.0, "imag", noise(shape, "imag") * 2.0 ** 20, 3)
