@@ -9,9 +9,9 @@
 // instructions: one issue slot for two lanes' arithmetic).
 //
 // Increments are carried times 2^kSplitShift, so that FP32's exponent range covers
-// fields from 2^-150 (below: the increments lose bits, and vanish under 2^-205) up to
-// kSplitMaxField = 2^67 in modulus; larger or non-finite values are the caller's to
-// detect (split3's tmax) and send through FP64.
+// values from 2^-150 (below: the increments lose bits, and vanish under 2^-182) up to 2^67 in
+// modulus.  Larger or non-finite values are the caller's to detect (split3's tmax), and so are
+// fields that are small as a whole (kIncTiny in gp_sweeps64.cu); both go through FP64.
 //
 // The error-free transformations are the published ones: TwoSum (Knuth, The Art of
 // Computer Programming 2, 4.2.2) and the FMA product residual; every operation is an
@@ -392,13 +392,13 @@ GP_HD Two second_difference(const Three& a, const Three& b, const Three& c) {
 
 // (h + l) 2^(k - kSplitShift) as an FP64 number, of a two_norm'ed number: l is added to
 // the significand of h in units of its FP64 ulp, and because it never points back below
-// h the unit is right at powers of two as well.
+// h the unit is right at powers of two as well.  A subnormal h counts as zero.
 GP_HD double to_double(float h, float l, int k) {
   const uint32_t a = f_bits(h);
   // |l| in units of 2^(E - 52), E the exponent of h
   const float q = bits_f(0x7f000000u - (a & 0x7f800000u));
   const uint32_t ci = (uint32_t)round_int(fabsf((l * q) * 0x1p52f));
-  const uint32_t off = (a << 1) == 0u ? 0u : (uint32_t)(kSplitOff + (k << 20));
+  const uint32_t off = (a & 0x7f800000u) == 0u ? 0u : (uint32_t)(kSplitOff + (k << 20));
   const uint32_t top = (uint32_t)((int32_t)a >> 3) & 0x8fffffffu;   // sign, exponent and leading significand
   const uint64_t w = (((uint64_t)top << 32) | (uint64_t)(a << 29)) + (((uint64_t)off << 32) | ci);
   return from_words((uint32_t)(w >> 32), (uint32_t)w);

@@ -462,6 +462,10 @@ constexpr int kIncSms = 152;     // SMs of a GB300
 
 // Noise is looked for in values above 2^-10 of the field's largest (noise below that, in
 // the far tails, adds nothing to the field's error); amax: its high word.
+// Fields of that size and less are not for FP32's exponent range (gp_split.cuh): increments
+// lose bits from 2^-150, which leaves 2^60 for the field's smaller values and for what a step
+// changes.  They are computed in FP64 throughout.
+constexpr int kIncTiny = (1023 - 90) << 20;
 __device__ __forceinline__ float inc_floor(int amax) {
   const int t = addmax0(amax, -kSplitOff);
   return t >= kSplitTooBig ? 0.f : bits_f((uint32_t)t << 3) * 0x1p-10f;
@@ -532,11 +536,11 @@ __device__ __forceinline__ double2 get_d2(const float4* q) { return *reinterpret
 // j0 + kIncL (zero outside the line).  io.load(u): v again for the final addition;
 // io.store(u, v, c): the increment c of point j0 + u (j0 + u < n); io.rd(j): v of any point
 // of the line (FP64 path).  Every thread of the block must call it; `on`: the thread owns a
-// segment.
+// segment; tiny (the same in every thread): the FP64 path.
 template <bool CPLX, class IO>
 __device__ __forceinline__ void inc_segment(const IncRho<CPLX>& rho, float4* slot, int TS, float4* carry,
                                             int T, int X, int sg, int nseg, int j0, int n, bool on,
-                                            double2 before, double2 after, float least, IO& io) {
+                                            double2 before, double2 after, float least, bool tiny, IO& io) {
   int tmax = 0;
   // noise: somewhere sampled, the second difference is opposite in sign to v and larger
   // than the values (complex: the moduli) around it and than least
@@ -566,7 +570,7 @@ __device__ __forceinline__ void inc_segment(const IncRho<CPLX>& rho, float4* slo
   // accuracy, and most blocks of a turbulent field would go: 101 x 77 x 53 complex, 20
   // steps late in a run 2281 us, with half a warp 1351)
   const bool noise = __popc(__ballot_sync(0xffffffffu, on && noisy)) >= 16;
-  if (!__syncthreads_or(noise || (on && tmax >= kSplitTooBig))) {
+  if (!__syncthreads_or(tiny || noise || (on && tmax >= kSplitTooBig))) {
     // carry out to the next segment: the tail of s; the first segment also starts itself
     put_two(carry, inc_carry(rho, [&](int k) { return get_two(slot + (kIncL - 1 - k) * TS); }));
     Prod pr = prod_zero();
@@ -689,10 +693,11 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_inc64(const __grid_consta
   cp_async_commit();
   const double2 before = io.rd(j0 - 1), after = io.rd(j0 + kIncL);
   const IncRho<CPLX> rho(p);
-  const float least = inc_floor(AXIS == 1 ? amax_of_step(p.inc_amax) : p.inc_amax[kAmaxNow]);
+  const int amax = AXIS == 1 ? amax_of_step(p.inc_amax) : p.inc_amax[kAmaxNow];
   if (AXIS == 1 && blockIdx.x == 0 && tid == 0) amax_end_step(p.inc_amax);
   cp_async_wait<0>();
-  inc_segment<CPLX>(rho, slot, T, carry, T, X, sg, nseg, j0, n, io.on, before, after, least, io);
+  inc_segment<CPLX>(rho, slot, T, carry, T, X, sg, nseg, j0, n, io.on, before, after, inc_floor(amax),
+                    amax < kIncTiny, io);
   if constexpr (NORM) norm_finish(io.acc, p.partials, p.counter, gridDim.x, blockIdx.x, p.scale_out,
                                   p.status, p.dV);
 }
@@ -706,7 +711,8 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_inc64(const __grid_consta
 // row's times the pending factor, less 1; v' = v + v e: real, e as FP64 and one DFMA; complex,
 // v e in two-part FP32 and one DADD per part.  q is skipped where every lane of the warp has |y| < 2^-56, and taken from short or
 // long Taylor sums by the size of y; a warp with |y| > 1/8, |E| > 1/4 (where 1 + E in two
-// parts would lose to FP64) or values out of range computes the substep in FP64.
+// parts would lose to FP64) or values out of range, and every warp of a tiny field, computes
+// the substep in FP64.
 // Measured at 240 x 200 x 160 with the solve: 284 us (k_sweep_x64 at its shortest
 // polynomial; 620 us where the density calls for the longer one) -> 92 us, complex 686
 // -> 194 us.
@@ -787,6 +793,7 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
   const int par = amax_parity(p.inc_amax, blockIdx.x == 0 && tid == 0);
   __syncthreads();
   const float least = inc_floor(head_now);
+  const bool tiny = head_now < kIncTiny;
   const double spre = head_d[0], s = head_d[1], cy = head_d[2];
   const bool pre = __double2hiint(spre) != 0x3ff00000 || __double2loint(spre) != 0;
   const bool pw = p.pw != 0;
@@ -858,7 +865,7 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
         } else {
           e = two_add(get_two(rc + 2), prod_add(two_mul(exi, get_two(rc + 1)), two_mul(ex, get_two(rc))));
         }
-        bool ok = fmaxf(fabsf(e.h.x), fabsf(e.h.y)) <= kIncBigE;
+        bool ok = !tiny && fmaxf(fabsf(e.h.x), fabsf(e.h.y)) <= kIncBigE;
         int tmax = 0;
         Two V;
         if (CPLX) {
@@ -965,7 +972,8 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
     if (io.on && sg > 0) before = get_d2(slots + tid - X + (kIncL - 1) * TS);
     if (io.on && sg + 1 < nseg) after = get_d2(slots + tid + X);
     __syncthreads();
-    inc_segment<CPLX>(rho, slots + tid, TS, carry, T, X, sg, nseg, j0, nx, io.on, before, after, least, io);
+    inc_segment<CPLX>(rho, slots + tid, TS, carry, T, X, sg, nseg, j0, nx, io.on, before, after, least,
+                      tiny, io);
   }
   __syncthreads();
   for (int ch = 0; ch < nchunk; ++ch) {

@@ -80,3 +80,18 @@ def test_noise_in_a_field_that_has_fallen(P, shape):
     normalised size at the start: what counts as noise follows the field down."""
     h = 0.05   # (a trap whose factor stays near 1 over the whole grid)
     check(P, shape, h, 0.1 * h * h, 0.0, "imag", noise(shape, "imag") * 2.0 ** 20, 3)
+
+
+@pytest.mark.parametrize("mode", ["imag", "real"])
+@pytest.mark.parametrize("amp", [2.0 ** -85, 2.0 ** -95, 1e-45, 1e-60, 1e-150])
+@pytest.mark.parametrize("shape", [(45, 38, 34), (64, 50, 1)])
+def test_fields_of_very_small_amplitude(P, mode, amp, shape):
+    """At the edge of FP32's exponent range and far below it; in imaginary time the step after
+    the first is of normal size again."""
+    h, steps = 0.2, 2
+    x, y, z = ((np.arange(n) - 0.5 * (n - 1)) * h for n in shape)
+    f = amp * np.exp(-0.3 * (z[:, None, None] ** 2 + y[None, :, None] ** 2 + x[None, None, :] ** 2))
+    f = f * (1 + 0.2 * np.cos(1.3 * x + 0.4)[None, None, :] * np.cos(0.7 * y)[None, :, None])
+    if mode == "real":
+        f = f * np.exp(0.4j * np.sin(x + 0.2))[None, None, :]
+    check(P, shape, h, 0.004, 0.0, mode, f, steps)
