@@ -262,8 +262,9 @@ GP_HD Two two_const_fma(float2 ch, float2 cl, const Two& y, float2 a) {
   p.l = fma2(y.l, a, fma2(y.h, a, mul2(p.h, f2(-1.f))));
   return two_add(two_scalar(ch, cl), p);
 }
-// exp(-y) - 1 for 0 <= |y| <= 1/16 (Taylor; the terms from y^5 on, below 2^-27, in FP32)
-GP_HD Two two_expm1_neg(const Two& y) {
+// (exp(-y) - 1 + y) / y^2 for |y| <= 1/16 (Taylor; the terms of exp from y^5 on, below 2^-27,
+// in FP32)
+GP_HD Two two_exp_series(const Two& y) {
   const float2 y1 = y.h;
   float2 a = fma2(y1, f2(1.f / 40320.f), f2(-1.f / 5040.f));
   a = fma2(y1, a, f2(1.f / 720.f));
@@ -271,11 +272,14 @@ GP_HD Two two_expm1_neg(const Two& y) {
   // 1/24, 1/6 as an FP32 pair
   Two w = two_const_fma(f2(1.f / 24.f), f2((float)(1.0 / 24.0 - (double)(1.f / 24.f))), y, a);
   w = two_add(two_scalar(f2(-1.f / 6.f), f2((float)(-(1.0 / 6.0 - (double)(1.f / 6.f))))), two_mul(y, w));
-  w = two_add(two_scalar(f2(0.5f), f2(0.f)), two_mul(y, w));
-  w = two_add(two_scalar(f2(-1.f), f2(0.f)), two_mul(y, w));
-  return two_mul(y, w);
+  return two_add(two_scalar(f2(0.5f), f2(0.f)), two_mul(y, w));
 }
-// The same for |y| <= 2^-9: y^3 and higher terms (below 2^-29) in FP32
+// exp(-y) - 1, and the same without its leading term, exp(-y) - 1 + y
+GP_HD Two two_expm1_neg(const Two& y) {
+  return two_mul(y, two_add(two_scalar(f2(-1.f), f2(0.f)), two_mul(y, two_exp_series(y))));
+}
+GP_HD Two two_expm1_neg_rest(const Two& y) { return two_mul(y, two_mul(y, two_exp_series(y))); }
+// exp(-y) - 1 for |y| <= 2^-9: y^3 and higher terms (below 2^-29) in FP32
 GP_HD Two two_expm1_neg_small(const Two& y) {
   const float2 y1 = y.h, y2 = mul2(y1, y1);
   const float2 a = fma2(y1, fma2(y1, f2(-1.f / 120.f), f2(1.f / 24.f)), f2(-1.f / 6.f));
@@ -294,20 +298,27 @@ GP_HD Two two_cmul(const Two& a, const Two& b) {
   const Two ai = two_scalar(f2(-a.h.y, a.h.y), f2(-a.l.y, a.l.y));
   return two_add(two_mul(ar, b), two_mul(ai, two_swap(b)));
 }
-// (cos y - 1, -sin y) for |y| <= 1/16, both lanes of y the same (Taylor in z = y^2; the
+// (cos y - 1, 1 - sin y / y) for |y| <= 1/16, both lanes of y the same (Taylor in z = y^2; the
 // terms from z^3 / 720 and y z^3 / 5040 on in FP32)
-GP_HD Two two_cis_neg_m1(const Two& y) {
+GP_HD Two two_cis_series(const Two& y) {
   const Two z = two_mul(y, y);
   const float2 a = fma2(z.h, f2(1.f / 40320.f, 0.f), f2(-1.f / 720.f, 1.f / 5040.f));
   Two w = two_const_fma(f2(1.f / 24.f, -1.f / 120.f),
                         f2((float)(1.0 / 24.0 - (double)(1.f / 24.f)), (float)(-(1.0 / 120.0 - (double)(1.f / 120.f)))),
                         z, a);
   w = two_add(two_scalar(f2(-0.5f, 1.f / 6.f), f2(0.f, (float)(1.0 / 6.0 - (double)(1.f / 6.f)))), two_mul(z, w));
-  const Two c = two_mul(z, w);
-  const Two m = two_mul(y, two_add(two_scalar(f2(-1.f), f2(0.f)), c));
+  return two_mul(z, w);
+}
+// (cos y - 1, -sin y), and the same without its leading term, (cos y - 1, y - sin y)
+GP_HD Two two_cis_neg_m1(const Two& y) {
+  const Two c = two_cis_series(y), m = two_mul(y, two_add(two_scalar(f2(-1.f), f2(0.f)), c));
   return two_scalar(f2(c.h.x, m.h.y), f2(c.l.x, m.l.y));
 }
-// The same for |y| <= 2^-10: z^2 and y z terms (below 2^-32) in FP32
+GP_HD Two two_cis_neg_rest(const Two& y) {
+  const Two c = two_cis_series(y), m = two_mul(y, c);
+  return two_scalar(f2(c.h.x, m.h.y), f2(c.l.x, m.l.y));
+}
+// (cos y - 1, -sin y) for |y| <= 2^-10: z^2 and y z terms (below 2^-32) in FP32
 GP_HD Two two_cis_neg_m1_small(const Two& y) {
   const Two z = two_mul(y, y);
   const float re = z.h.x, rel = z.l.x;

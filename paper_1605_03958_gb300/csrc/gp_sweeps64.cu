@@ -471,6 +471,13 @@ __device__ __forceinline__ float inc_floor(int amax) {
   return t >= kSplitTooBig ? 0.f : bits_f((uint32_t)t << 3) * 0x1p-10f;
 }
 
+// A power of two that takes values times 2^kSplitShift to units of the field's largest (amax:
+// its high word): that becomes 1 to 2.
+__device__ __forceinline__ float inc_unit(int amax) {
+  const int t = min(addmax0(amax, -kSplitOff), 253 << 20);
+  return bits_f((uint32_t)(254 - (t >> 20)) << 23);
+}
+
 template <bool CPLX> struct IncRho;
 template <> struct IncRho<false> {
   Coef r;
@@ -709,10 +716,19 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_inc64(const __grid_consta
 //   e = E + (1 + E) q,   E = ex + er + ex er,   q = exp(-y) - 1 (cis(-y) - 1),
 // ex the column's factor less 1 (two-part table, from expm1 / sin^2 in FP64), er the
 // row's times the pending factor, less 1; v' = v + v e: real, e as FP64 and one DFMA; complex,
-// v e in two-part FP32 and one DADD per part.  q is skipped where every lane of the warp has |y| < 2^-56, and taken from short or
-// long Taylor sums by the size of y; a warp with |y| > 1/8, |E| > 1/4 (where 1 + E in two
-// parts would lose to FP64) or values out of range, and every warp of a tiny field, computes
-// the substep in FP64.
+// v e in two-part FP32 and one DADD per part.  q is skipped where every lane of the warp has
+// |y| < 2^-56, and taken from short or long Taylor sums by the size of y.
+//
+// 48 bits of e are 53 of v' as long as e is small.  Relative error against quadruple precision,
+// two-part / FP64 products (1e-16), at |E| = 1e-3, 1/64, 0.1, 0.28: real 0.6 / 0.9, 0.8 / 0.9, 2.7 /
+// 1.0, 6.6 / 1.0, complex 0.6 / 1.1, 1.0 / 1.1, 5.0 / 1.1, 17 / 1.1; at y = 1/128, 0.02, 0.1: 0.7 /
+// 1.0, 1.2 / 1.1, 8.6 / 1.1 and (1/256) 0.7 / 1.0, 1.3 / 1.0, 5.4 / 1.2.  So
+//   |y| from kIncY to 1/16: q's leading term (-y, -i y) in FP64, four operations per real
+//     value and seven per complex one, the rest of e as before;
+//   |E| > kIncE: the substep in FP64, except for |E| up to kIncBigE where the value is so small
+//     against the field's largest that its error stays below 2^-10 of such an |E|'s there;
+//   |y| > 1/16, values out of range, a tiny field: in FP64,
+// each for a warp as a whole.
 // Measured at 240 x 200 x 160 with the solve: 284 us (k_sweep_x64 at its shortest
 // polynomial; 620 us where the density calls for the longer one) -> 92 us, complex 686
 // -> 194 us.
@@ -723,6 +739,8 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_inc64(const __grid_consta
 // (as the y / z kernel; the increments replace the slots); lanes along the rows again
 // for u = v' + c.
 constexpr float kIncBigE = 0.25f;
+constexpr float kIncE = 1.f / 64;
+template <bool CPLX> constexpr float kIncY = CPLX ? 1.f / 256 : 1.f / 128;
 
 // v' in FP64 (f: the folded factor times the trap factors; real, complex)
 __device__ __forceinline__ double pointwise64(double v, double f, double cy) {
@@ -753,6 +771,27 @@ __device__ __forceinline__ double2 pointwise64(double2 v, double2 f, double cy) 
     sincos(th, &sn, &cs);
   }
   return cmul(cmul(v, f), make_double2(cs, -sn));
+}
+
+// The real pair's or complex value's v' with y's leading term in FP64 (|y| <= 1/16); e: E, V: v
+// in two parts, cyc: cy.
+template <bool CPLX> __device__ __forceinline__ double2 pointwise_lead(double2 v, Two e, const Two& V, const Coef& cyc, double cy) {
+  const Two h = two_scalar(mul2(V.h, f2(0x1p-56f)), mul2(V.l, f2(0x1p-56f)));
+  Two d = two_mul(h, h);
+  if (CPLX) d = two_add(d, two_swap(d));
+  const Two y = prod_two(two_mul(cyc, d));
+  const Two rest = CPLX ? two_cis_neg_rest(y) : two_expm1_neg_rest(y);
+  const Two q = two_add(rest, CPLX ? two_scalar(f2(0.f, -y.h.y), f2(0.f, -y.l.y)) : two_neg(y));
+  e = two_add(two_add(e, rest), CPLX ? two_cmul(e, q) : two_mul(e, q));
+  const Two c = two_norm(CPLX ? two_cmul(V, e) : e);
+  const int k = CPLX ? 0 : kSplitShift;
+  const double2 w = make_double2(to_double(c.h.x, c.l.x, k), to_double(c.h.y, c.l.y, k));
+  if constexpr (CPLX) {
+    const double th = cy * fma(v.x, v.x, v.y * v.y);
+    return make_double2(v.x + fma(th, v.y, w.x), v.y + fma(-th, v.x, w.y));
+  } else {
+    return make_double2(fma(v.x, fma(-cy * v.x, v.x, w.x), v.x), fma(v.y, fma(-cy * v.y, v.y, w.y), v.y));
+  }
 }
 
 template <bool CPLX>
@@ -794,6 +833,7 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
   __syncthreads();
   const float least = inc_floor(head_now);
   const bool tiny = head_now < kIncTiny;
+  const float unit = inc_unit(head_now);
   const double spre = head_d[0], s = head_d[1], cy = head_d[2];
   const bool pre = __double2hiint(spre) != 0x3ff00000 || __double2loint(spre) != 0;
   const bool pw = p.pw != 0;
@@ -844,6 +884,14 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
       return con && r < rows && GP_IN(at0 + (long long)r * P + cv, nall, p.status)
                  ? field[(size_t)r * P + cv] : zero;
     };
+    auto factor = [&](const float4* rc) {   // E of the column and a row
+      if constexpr (!CPLX) {
+        const float4 f = rc[0];
+        return two_add(two_scalar(f2(f.z), f2(f.w)), two_mul(ex, two_scalar(f2(f.x), f2(f.y))));
+      } else {
+        return two_add(get_two(rc + 2), prod_add(two_mul(exi, get_two(rc + 1)), two_mul(ex, get_two(rc))));
+      }
+    };
     double2 nxt = fetch(ro);
     for (int q = 0; q < rounds; ++q) {   // (full rounds: every lane takes part in the votes)
       const int r = ro + q * grp;
@@ -858,15 +906,12 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
       vmax = imax(vmax, vm);
       if (work) {
         const float4* rc = rowc + (CPLX ? 3 : 1) * (live ? r : 0);
-        Two e;
-        if constexpr (!CPLX) {
-          const float4 f = rc[0];
-          e = two_add(two_scalar(f2(f.z), f2(f.w)), two_mul(ex, two_scalar(f2(f.x), f2(f.y))));
-        } else {
-          e = two_add(get_two(rc + 2), prod_add(two_mul(exi, get_two(rc + 1)), two_mul(ex, get_two(rc))));
-        }
-        bool ok = !tiny && fmaxf(fabsf(e.h.x), fabsf(e.h.y)) <= kIncBigE;
+        Two e = factor(rc);
+        const float em = fmaxf(fabsf(e.h.x), fabsf(e.h.y));
+        const float size = bits_f((uint32_t)min(addmax0(vm, -kSplitOff), 253 << 20) << 3) * unit;
+        bool ok = !tiny && (em <= kIncE || (em <= kIncBigE && em * size <= 0x1p-10f));
         int tmax = 0;
+        float ym = 0.f;
         Two V;
         if (CPLX) {
           V = split2(v.x, v.y, &tmax);
@@ -878,24 +923,17 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
           const Two h = two_scalar(mul2(V.h, f2(0x1p-56f)), mul2(V.l, f2(0x1p-56f)));
           Two d = two_mul(h, h);
           if (CPLX) d = two_add(d, two_swap(d));   // re^2 + im^2 in both lanes
-          Two y = prod_two(two_mul(cyc, d));
-          const float ym = fmaxf(fabsf(y.h.x), fabsf(y.h.y));
-          ok = ok && ym <= 0.125f && tmax < kSplitTooBig;
+          const Two y = prod_two(two_mul(cyc, d));
+          ym = fmaxf(fabsf(y.h.x), fabsf(y.h.y));
+          ok = ok && tmax < kSplitTooBig;
           Two qv;
-          if (__all_sync(0xffffffffu, ym <= 0x1p-10f || !ok)) {
+          if (__all_sync(0xffffffffu, ym <= 0x1p-10f || !ok))
             qv = CPLX ? two_cis_neg_m1_small(y) : two_expm1_neg_small(y);
-          } else {
-            const int halvings = __all_sync(0xffffffffu, ym <= (CPLX ? 0.0625f : 0.03125f) || !ok) ? 0
-                                 : __all_sync(0xffffffffu, ym <= (CPLX ? 0.125f : 0.0625f) || !ok) ? 1 : 2;
-            const float sc = halvings == 0 ? 1.f : halvings == 1 ? 0.5f : 0.25f;
-            y = two_scalar(mul2(y.h, f2(sc)), mul2(y.l, f2(sc)));
+          else
             qv = CPLX ? two_cis_neg_m1(y) : two_expm1_neg(y);
-            for (int k = 0; k < halvings; ++k)
-              qv = two_add(two_scalar(add2(qv.h, qv.h), add2(qv.l, qv.l)), CPLX ? two_cmul(qv, qv) : two_mul(qv, qv));
-          }
           e = two_add(two_add(e, qv), CPLX ? two_cmul(e, qv) : two_mul(e, qv));
         }
-        if (__all_sync(0xffffffffu, ok || !live)) {
+        if (__all_sync(0xffffffffu, (ok && ym <= kIncY<CPLX>) || !live)) {
           if constexpr (CPLX) {
             const Two c = two_norm(two_cmul(V, e));
             v.x += to_double(c.h.x, c.l.x, 0);
@@ -905,6 +943,8 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
             v.x = fma(v.x, to_double(c.h.x, c.l.x, kSplitShift), v.x);
             v.y = fma(v.y, to_double(c.h.y, c.l.y, kSplitShift), v.y);
           }
+        } else if (__all_sync(0xffffffffu, (ok && ym <= 0.0625f) || !live)) {
+          v = pointwise_lead<CPLX>(v, factor(rc), V, cyc, cy);
         } else if (live) {
           const double c2 = pw ? cy : 0.0;
           // |y| < 2^-56: the factor alone (the far field, where |E| is large and v small: two

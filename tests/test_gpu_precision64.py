@@ -95,3 +95,18 @@ def test_fields_of_very_small_amplitude(P, mode, amp, shape):
     if mode == "real":
         f = f * np.exp(0.4j * np.sin(x + 0.2))[None, None, :]
     check(P, shape, h, 0.004, 0.0, mode, f, steps)
+
+
+@pytest.mark.parametrize("mode", ["imag", "real"])
+@pytest.mark.parametrize("y,h", [(0.006, 0.05), (0.02, 0.05), (0.05, 0.05), (0.1, 0.05), (0.4, 0.05),
+                                 (0.001, 0.2), (0.001, 0.3), (0.001, 0.45), (0.02, 0.3)])
+@pytest.mark.parametrize("shape", [(45, 38, 34), (64, 50, 1)])
+def test_substep_of_large_density_or_trap(P, shape, y, h, mode):
+    """Fields spread over the whole box (half waves that vanish at its walls): dt g |psi|^2 up to
+    y, trap factors from near 1 (h = 0.05) to exp(-2) and beyond at the walls (h = 0.45)."""
+    s = [np.sin(np.pi * (np.arange(n) + 1) / (n + 1)) if n > 1 else np.ones(1) for n in shape]
+    f = 0.3 * s[2][:, None, None] * s[1][None, :, None] * s[0][None, None, :]
+    if mode == "real":
+        f = f * np.exp(0.4j * np.sin(np.arange(shape[0]) * 0.1))[None, None, :]
+    dt = 0.1 * h * h
+    check(P, shape, h, dt, y / (0.09 * dt), mode, f, 1)
