@@ -105,6 +105,7 @@ struct SweepParams {
   int inc_x, inc_seg;    // inc_x = 0: not used
   double rho[2];
   float rho_f[4];
+  float inc_rough;       // rms(v)^2 / rms(s)^2 up to which a block is rough, s the second difference
   int inc_quiet;         // x: high word of |v| below which the nonlinear term is nothing
   int* inc_amax;         // FP64: words of the field's largest value (kAmax*)
   const void* inc_ex;    // x: trap factor along x less 1, two-part FP32, per 16-byte vector of a row:

@@ -438,12 +438,15 @@ __global__ void __launch_bounds__(kLineThreads) k_sweep_line64(const __grid_cons
 // 18 per complex one in k_sweep_line64.  Measured at 240 x 200 x 160 (GB300, event-timed
 // launches): y 80 -> 44 us, z with its norm 106 -> 59 us; complex y 245 -> 91 us, z 290 ->
 // 83 us.  Now bound by issue (2.2-2.4 of 4 instructions per clock, 116 per real point,
-// 260 per complex one) and the FP64 pipe (34-54 %).  Accuracy: on smooth lines
-// s is exact and the increment's error is far below the final rounding (relative L2 of a
-// sweep against quadruple precision, a = 0.025: 4.8e-17, the rounding of u alone, where
-// the FP64 recurrence has 1.2e-16).  On a line of grid-scale noise s has no spare bits
-// left and two FP32 parts would lose to FP64 (4.2e-16), so a block that sees such values
-// (or any too large for FP32's range, or non-finite) evaluates its lines in FP64.
+// 260 per complex one) and the FP64 pipe (34-54 %).
+//
+// Accuracy: s is exact and the increment's 48 bits are far below the final rounding as long as
+// the increment is small against v.  Relative L2 error of a sweep against quadruple precision
+// is about the root of (4e-17)^2, the rounding of u, plus (1e-14 |a| rms(s) / rms(v))^2: waves
+// of 64 points at a = 0.025, k h = 0.3: 5.9e-17 (the FP64 recurrence 1.0e-16), 0.6: 9.7e-17,
+// 0.9: 1.5e-16, white noise 4.5e-16 (1.2e-16); complex ones the same (recurrence 1.3e-16).  So
+// a block whose points have |a| rms(s) > rms(v) / 128 evaluates its lines in FP64 (noise
+// 5.7e-17), and so does one with values too large for FP32's range or not finite.
 //
 // A thread owns one 16-byte vector position (two real x or one complex x) and a segment of
 // 16 points of the line; the block holds whole lines (all segments of inc_x positions),
@@ -459,17 +462,12 @@ constexpr int kIncH = 12;        // terms of a carry
 constexpr int kIncNear = 6;      // of those, the near ones in two-part arithmetic
 constexpr int kIncThreads = 256; // most threads per block
 constexpr int kIncSms = 152;     // SMs of a GB300
+constexpr double kIncRough = 128.0;  // a block is rough from rms(v) / rms(s) = kIncRough |a|
 
-// Noise is looked for in values above 2^-10 of the field's largest (noise below that, in
-// the far tails, adds nothing to the field's error); amax: its high word.
 // Fields of that size and less are not for FP32's exponent range (gp_split.cuh): increments
 // lose bits from 2^-150, which leaves 2^60 for the field's smaller values and for what a step
 // changes.  They are computed in FP64 throughout.
 constexpr int kIncTiny = (1023 - 90) << 20;
-__device__ __forceinline__ float inc_floor(int amax) {
-  const int t = addmax0(amax, -kSplitOff);
-  return t >= kSplitTooBig ? 0.f : bits_f((uint32_t)t << 3) * 0x1p-10f;
-}
 
 // A power of two that takes values times 2^kSplitShift to units of the field's largest (amax:
 // its high word): that becomes 1 to 2.
@@ -543,15 +541,16 @@ __device__ __forceinline__ double2 get_d2(const float4* q) { return *reinterpret
 // j0 + kIncL (zero outside the line).  io.load(u): v again for the final addition;
 // io.store(u, v, c): the increment c of point j0 + u (j0 + u < n); io.rd(j): v of any point
 // of the line (FP64 path).  Every thread of the block must call it; `on`: the thread owns a
-// segment; tiny (the same in every thread): the FP64 path.
+// segment; unit: inc_unit; limit: inc_rough; tiny: the FP64 path (these the same in every thread).
 template <bool CPLX, class IO>
 __device__ __forceinline__ void inc_segment(const IncRho<CPLX>& rho, float4* slot, int TS, float4* carry,
                                             int T, int X, int sg, int nseg, int j0, int n, bool on,
-                                            double2 before, double2 after, float least, bool tiny, IO& io) {
+                                            double2 before, double2 after, float unit, float limit, bool tiny, IO& io) {
   int tmax = 0;
-  // noise: somewhere sampled, the second difference is opposite in sign to v and larger
-  // than the values (complex: the moduli) around it and than least
-  bool noisy = false;
+  // sums of |s|^2 and |v|^2 over half of the block's points (pairs of neighbours: no wave is
+  // missed at its zeros), in units of the field's largest value; each value counts as 2^-10 at
+  // least (noise below that, in the far tails, adds nothing to the field's error)
+  float2 rough = f2(0.f), mass = f2(kIncL / 2 * 0x1p-20f);
   {
     const double2 v0 = get_d2(slot);
     Three a = split3(before.x, before.y, &tmax), b = split3(v0.x, v0.y, &tmax);
@@ -561,23 +560,28 @@ __device__ __forceinline__ void inc_segment(const IncRho<CPLX>& rho, float4* slo
       const Three c = split3(vn.x, vn.y, &tmax);
       const Two s = second_difference(a, b, c);
       put_two(slot + u * TS, s);
-      if (u % 4 == 2) {
-        float lx = fmaxf(least, fmaxf(fabsf(a.h.x), fmaxf(fabsf(b.h.x), fabsf(c.h.x))));
-        float ly = fmaxf(least, fmaxf(fabsf(a.h.y), fmaxf(fabsf(b.h.y), fabsf(c.h.y))));
-        if (CPLX) lx = ly = fmaxf(lx, ly);
-        noisy = noisy || (fabsf(s.h.x) > lx && s.h.x * b.h.x < 0.f) ||
-               (fabsf(s.h.y) > ly && s.h.y * b.h.y < 0.f);
+      if (u % 4 >= 2) {
+        const float2 sh = mul2(s.h, f2(unit)), vh = mul2(b.h, f2(unit));
+        if (j0 + u < n) rough = fma2(sh, sh, rough);
+        mass = fma2(vh, vh, mass);
       }
       a = b;
       b = c;
     }
   }
-  // values out of range, or noise at half the segments of a warp: the block computes in FP64
-  // (one noisy segment is not enough: a field with fine structure here and there keeps its
-  // accuracy, and most blocks of a turbulent field would go: 101 x 77 x 53 complex, 20
-  // steps late in a run 2281 us, with half a warp 1351)
-  const bool noise = __popc(__ballot_sync(0xffffffffu, on && noisy)) >= 16;
-  if (!__syncthreads_or(tiny || noise || (on && tmax >= kSplitTooBig))) {
+  // a tiny field, values out of range or a rough block (see kIncRough): in FP64
+  __shared__ float2 part[kIncThreads / 32];
+  {
+    float2 sum = on ? f2(rough.x + rough.y, mass.x + mass.y) : f2(0.f);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      sum = add2(sum, f2(__shfl_xor_sync(0xffffffffu, sum.x, o), __shfl_xor_sync(0xffffffffu, sum.y, o)));
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sum;
+  }
+  const bool big = __syncthreads_or(tiny || (on && tmax >= kSplitTooBig));
+  float2 sum = part[0];
+  for (unsigned int w = 1; w < blockDim.x / 32; ++w) sum = add2(sum, part[w]);
+  if (!big && sum.x * limit < sum.y) {
     // carry out to the next segment: the tail of s; the first segment also starts itself
     put_two(carry, inc_carry(rho, [&](int k) { return get_two(slot + (kIncL - 1 - k) * TS); }));
     Prod pr = prod_zero();
@@ -703,8 +707,8 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_inc64(const __grid_consta
   const int amax = AXIS == 1 ? amax_of_step(p.inc_amax) : p.inc_amax[kAmaxNow];
   if (AXIS == 1 && blockIdx.x == 0 && tid == 0) amax_end_step(p.inc_amax);
   cp_async_wait<0>();
-  inc_segment<CPLX>(rho, slot, T, carry, T, X, sg, nseg, j0, n, io.on, before, after, inc_floor(amax),
-                    amax < kIncTiny, io);
+  inc_segment<CPLX>(rho, slot, T, carry, T, X, sg, nseg, j0, n, io.on, before, after, inc_unit(amax),
+                    p.inc_rough, amax < kIncTiny, io);
   if constexpr (NORM) norm_finish(io.acc, p.partials, p.counter, gridDim.x, blockIdx.x, p.scale_out,
                                   p.status, p.dV);
 }
@@ -831,7 +835,6 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
   }
   const int par = amax_parity(p.inc_amax, blockIdx.x == 0 && tid == 0);
   __syncthreads();
-  const float least = inc_floor(head_now);
   const bool tiny = head_now < kIncTiny;
   const float unit = inc_unit(head_now);
   const double spre = head_d[0], s = head_d[1], cy = head_d[2];
@@ -1012,8 +1015,8 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
     if (io.on && sg > 0) before = get_d2(slots + tid - X + (kIncL - 1) * TS);
     if (io.on && sg + 1 < nseg) after = get_d2(slots + tid + X);
     __syncthreads();
-    inc_segment<CPLX>(rho, slots + tid, TS, carry, T, X, sg, nseg, j0, nx, io.on, before, after, least,
-                      tiny, io);
+    inc_segment<CPLX>(rho, slots + tid, TS, carry, T, X, sg, nseg, j0, nx, io.on, before, after,
+                      unit, p.inc_rough, tiny, io);
   }
   __syncthreads();
   for (int ch = 0; ch < nchunk; ++ch) {
@@ -1103,6 +1106,7 @@ bool inc64_setup(int axis, SweepParams* p, std::complex<double> a, bool complex_
   if (axis == 0) tiles = (tiles + kIncSms - 1) / kIncSms * kIncSms;
   p->inc_seg = nseg;
   p->inc_x = (nvec + tiles - 1) / tiles;
+  p->inc_rough = (float)(kIncRough * kIncRough * std::norm(a));
   const std::complex<double> r = 2.0 * a / (1.0 + 2.0 * a + std::sqrt(1.0 + 4.0 * a));
   const double part[2] = {r.real(), r.imag()};
   for (int q = 0; q < 2; ++q) {
