@@ -54,13 +54,15 @@ void slot_geometry(const gp_params& p, SlotGeom* G) {
   G->pitch[0] = (int)align_up((size_t)p.nx, 4);
   G->pitch[1] = (int)align_up((size_t)p.nx, 2);
   G->field_bytes = std::max((size_t)G->pitch[0] * 4, (size_t)G->pitch[1] * 8) * rows;
-  // z blocks at the shortest run (one turn of the smallest ring, 7 points)
-  int mb = 0;
-  for (int m = 0; m < 2; ++m) {
-    const long long cols = (long long)((p.nx + (m ? 1 : 3)) / (m ? 2 : 4)) * p.ny;
-    const long long nseg = (p.nz + 6) / 7;
-    mb = std::max<int>(mb, (int)((cols * nseg + 127) / 128));
-  }
+  // z blocks of the real field (which store a norm partial each) at any half-width and runs
+  // setting the slot can be launched with
+  long long mb = 0;
+  for (int w : {3, 5, gpk::kBandHalfMax})
+    for (int turns = 1; turns <= 3; ++turns) {
+      int runs, run;
+      gpk::batch_tile_shape(p.nz, w, turns, true, &runs, &run);
+      mb = std::max(mb, gpk::batch_tile_blocks(p.nx, p.ny, p.nz, runs, run, false));
+    }
   size_t off = 0;
   G->off_field = off;
   off = align_up(off + G->field_bytes, kAlign);
@@ -319,15 +321,8 @@ int rebuild(gp_pool* P) {
     d.nz = S.prm.nz;
     d.pitch = S.G.pitch[m];
     for (int a = 1; a < 3; ++a) {
-      const int n = a == 1 ? d.ny : d.nz;
-      int turns = P->seg_turns;
-      gpk::batch_tile_shape(n, P->wl[m][a], turns, m == 0 && a == 2, &d.tile_runs[a], &d.tile_run[a]);
-      // one norm partial per z block must fit the slot's area (a single run always does)
-      while (m == 0 && a == 2 && turns > 1 &&
-             gpk::batch_tile_blocks(d.nx, d.ny, n, d.tile_runs[a], d.tile_run[a], false) > S.G.max_blocks_z) {
-        turns = std::min(turns, 3) - 1;
-        gpk::batch_tile_shape(n, P->wl[m][a], turns, m == 0 && a == 2, &d.tile_runs[a], &d.tile_run[a]);
-      }
+      gpk::batch_tile_shape(a == 1 ? d.ny : d.nz, P->wl[m][a], P->seg_turns, m == 0 && a == 2,
+                            &d.tile_runs[a], &d.tile_run[a]);
     }
     d.dtg = (float)(S.prm.dt * S.g);
     d.dV = S.prm.dx * S.prm.dy * S.prm.dz;
