@@ -595,18 +595,32 @@ __global__ void __launch_bounds__(128) k_density_partial(const FieldParams p, in
         }
       }
     } else {
-      // values are scaled by a power of two that takes the largest of the eight vectors to
-      // about 1, which keeps the squares in FP32's range
-      float m = 0.f;
+      // values are scaled by a power of two that takes the column's largest of the eight to 1..2,
+      // which keeps the squares in FP32's range (columns apart: one can lie far below another)
+      float m[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int q = 0; q < 8; ++q)
-        m = fmaxf(fmaxf(fmaxf(m, fabsf(v[q].x)), fmaxf(fabsf(v[q].y), fabsf(v[q].z))), fabsf(v[q].w));
-      const int ex = min(max((int)(__float_as_uint(m) >> 23), 30), 223);
-      const float2 sc = f2(__uint_as_float((unsigned int)(254 - ex) << 23));
+      for (int q = 0; q < 8; ++q) {
+        m[0] = fmaxf(m[0], fabsf(v[q].x));
+        m[1] = fmaxf(m[1], fabsf(v[q].y));
+        m[2] = fmaxf(m[2], fabsf(v[q].z));
+        m[3] = fmaxf(m[3], fabsf(v[q].w));
+      }
+      if (CPLX) {
+        m[0] = m[1] = fmaxf(m[0], m[1]);
+        m[2] = m[3] = fmaxf(m[2], m[3]);
+      }
+      int ex[4];
+      float sc[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        ex[i] = min(max((int)(__float_as_uint(m[i]) >> 23), 30), 223);
+        sc[i] = __uint_as_float((unsigned int)(254 - ex[i]) << 23);
+      }
       Two s0 = two_zero(), s1 = two_zero();
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        const float2 a = mul2(f2(v[q].x, v[q].y), sc), b = mul2(f2(v[q].z, v[q].w), sc);
+        const float2 a = mul2(f2(v[q].x, v[q].y), f2(sc[0], sc[1]));
+        const float2 b = mul2(f2(v[q].z, v[q].w), f2(sc[2], sc[3]));
         Two qa, qb;
         qa.h = mul2(a, a);
         qa.l = fma2(a, a, mul2(qa.h, f2(-1.f)));
@@ -621,15 +635,15 @@ __global__ void __launch_bounds__(128) k_density_partial(const FieldParams p, in
       }
       s0 = two_norm(s0);
       s1 = two_norm(s1);
-      const int k = kSplitShift + 2 * (ex - 127);
+      auto shift = [&](int i) { return kSplitShift + 2 * (ex[i] - 127); };
       if (fabsf(s0.h.x) + fabsf(s0.h.y) + fabsf(s1.h.x) + fabsf(s1.h.y) <= 1e30f) {
-        acc[0] += to_double(s0.h.x, s0.l.x, k);
+        acc[0] += to_double(s0.h.x, s0.l.x, shift(0));
         if (CPLX) {
-          acc[1 % W] += to_double(s1.h.x, s1.l.x, k);
+          acc[1 % W] += to_double(s1.h.x, s1.l.x, shift(2));
         } else {
-          acc[1 % W] += to_double(s0.h.y, s0.l.y, k);
-          acc[2 % W] += to_double(s1.h.x, s1.l.x, k);
-          acc[3 % W] += to_double(s1.h.y, s1.l.y, k);
+          acc[1 % W] += to_double(s0.h.y, s0.l.y, shift(1));
+          acc[2 % W] += to_double(s1.h.x, s1.l.x, shift(2));
+          acc[3 % W] += to_double(s1.h.y, s1.l.y, shift(3));
         }
       } else {   // infinities or NaN among the values
         for (int q = 0; q < 8; ++q) {
