@@ -552,15 +552,50 @@ __global__ void k_export(const FieldParams p, double* __restrict__ dst, int as_c
 
 // ------------------------------------------------------- integrated densities
 
+// Sums of squares of FP32 values below 4 in modulus, on the FP32 pipe and two at a time: the
+// square's two exact parts are cut at fixed binary places (adding and subtracting a constant
+// rounds to its grid: the error-free vector transformation of Rump, Ogita and Oishi's AccSum, SIAM
+// J. Sci. Comput. 31, 2008), so that sums of sixteen of the upper two cuts are exact, of 2^-16 and
+// 2^-36, and only the third, below 2^-32, rounds: 2^-56 of the largest square.
+struct Squares {
+  float2 h, m, l;
+};
+__device__ __forceinline__ float2 on_grid(float2 x, float c) { return add2(add2(x, f2(c)), f2(-c)); }
+__device__ __forceinline__ void add_square(Squares& t, float2 a) {
+  constexpr float kGrid1 = 192.f, kGrid2 = 0x1.8p-13f;
+  const float2 qh = mul2(a, a), ql = fma2(a, a, mul2(qh, f2(-1.f)));
+  const float2 h = on_grid(qh, kGrid1), rest = sub2(qh, h);
+  const float2 m = on_grid(rest, kGrid2), n = on_grid(ql, kGrid2);
+  t.h = add2(t.h, h);
+  t.m = add2(t.m, add2(m, n));
+  t.l = add2(t.l, add2(sub2(rest, m), sub2(ql, n)));
+}
+__device__ __forceinline__ void add_lanes(Squares& t) {   // both lanes: their sum
+  t.h = add2(t.h, f2(t.h.y, t.h.x));
+  t.m = add2(t.m, f2(t.m.y, t.m.x));
+  t.l = add2(t.l, f2(t.l.y, t.l.x));
+}
+// the exponent field of the power of two that values up to m are divided by: the largest is 1 to
+// 4 then (all subnormal: less, but their squares are multiples of 2^-44, and every sum is exact)
+__device__ __forceinline__ int square_exponent(float m) { return min((int)(__float_as_uint(m) >> 23), 253); }
+__device__ __forceinline__ float square_scale(int ex) { return __uint_as_float((unsigned int)(254 - ex) << 23); }
+__device__ __forceinline__ bool finite_sums(float2 h) { return fabsf(h.x) + fabsf(h.y) <= 1e30f; }
+// acc plus the sum of lane x (y) of values that were divided by 2^(ex - 127)
+__device__ __forceinline__ double add_sum(double acc, float h, float m, float l, int ex) {
+  const int k = kSplitShift + 2 * (ex - 127);
+  const Two n = two_norm(two_scalar(f2(h), f2(m)));
+  return (acc + to_double(n.h.x, n.l.x, k)) + to_double(l, 0.f, k);
+}
+
 // |psi|^2 summed along one direction, kDensSum terms per thread: chunk ch of the nsum
 // rows `step` elements apart, for every column and each of the rows_out starting rows
 // `out_step` apart; part[(ch rows_out + o) nx + i].  One 16-byte vector per thread and
-// row.  FP64 work is what the sums must not wait for (see k_observables_two): FP32 values
-// are squared and added in two FP32 parts, eight terms at a time (their errors, about 2^-50
-// of the eight, average out over a chunk's and the chunks' FP64 additions), then added
-// in FP64; FP64 values cost one or two FP64 operations each.  The factor is applied by
-// the final sum.  Measured (240 x 200 x 160 complex64, the whole call): 202-239 -> 45-55 us
-// per density, of which the kernels take 16-20 us.
+// row.  FP64 work is what the sums must not wait for (see k_observables_two): FP32 values are
+// squared and added eight at a time as Squares, then in FP64; FP64 values cost one or two
+// FP64 operations each.  The factor is applied by the final sum.  Error against extended
+// precision as of FP64 sums throughout, 2e-16 rms (in two parts, eight terms at a time, 0.6e-15..
+// 1.7e-15).  Measured (240 x 200 x 160 complex64, the whole call): 52-54 us per density (two parts
+// 45-55, FP64 sums 202-239).
 constexpr int kDensSum = 32;
 template <class R, bool CPLX>
 __global__ void __launch_bounds__(128) k_density_partial(const FieldParams p, int rows_out, size_t out_step,
@@ -613,37 +648,27 @@ __global__ void __launch_bounds__(128) k_density_partial(const FieldParams p, in
       float sc[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        ex[i] = min(max((int)(__float_as_uint(m[i]) >> 23), 30), 223);
-        sc[i] = __uint_as_float((unsigned int)(254 - ex[i]) << 23);
+        ex[i] = square_exponent(m[i]);
+        sc[i] = square_scale(ex[i]);
       }
-      Two s0 = two_zero(), s1 = two_zero();
+      Squares s0{f2(0.f), f2(0.f), f2(0.f)}, s1 = s0;
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        const float2 a = mul2(f2(v[q].x, v[q].y), f2(sc[0], sc[1]));
-        const float2 b = mul2(f2(v[q].z, v[q].w), f2(sc[2], sc[3]));
-        Two qa, qb;
-        qa.h = mul2(a, a);
-        qa.l = fma2(a, a, mul2(qa.h, f2(-1.f)));
-        qb.h = mul2(b, b);
-        qb.l = fma2(b, b, mul2(qb.h, f2(-1.f)));
-        s0 = two_add(s0, qa);
-        s1 = two_add(s1, qb);
+        add_square(s0, mul2(f2(v[q].x, v[q].y), f2(sc[0], sc[1])));
+        add_square(s1, mul2(f2(v[q].z, v[q].w), f2(sc[2], sc[3])));
       }
       if (CPLX) {
-        s0 = two_add(s0, two_swap(s0));
-        s1 = two_add(s1, two_swap(s1));
+        add_lanes(s0);
+        add_lanes(s1);
       }
-      s0 = two_norm(s0);
-      s1 = two_norm(s1);
-      auto shift = [&](int i) { return kSplitShift + 2 * (ex[i] - 127); };
-      if (fabsf(s0.h.x) + fabsf(s0.h.y) + fabsf(s1.h.x) + fabsf(s1.h.y) <= 1e30f) {
-        acc[0] += to_double(s0.h.x, s0.l.x, shift(0));
+      if (finite_sums(s0.h) && finite_sums(s1.h)) {
+        acc[0] = add_sum(acc[0], s0.h.x, s0.m.x, s0.l.x, ex[0]);
         if (CPLX) {
-          acc[1 % W] += to_double(s1.h.x, s1.l.x, shift(2));
+          acc[1 % W] = add_sum(acc[1 % W], s1.h.x, s1.m.x, s1.l.x, ex[2]);
         } else {
-          acc[1 % W] += to_double(s0.h.y, s0.l.y, shift(1));
-          acc[2 % W] += to_double(s1.h.x, s1.l.x, shift(2));
-          acc[3 % W] += to_double(s1.h.y, s1.l.y, shift(3));
+          acc[1 % W] = add_sum(acc[1 % W], s0.h.y, s0.m.y, s0.l.y, ex[1]);
+          acc[2 % W] = add_sum(acc[2 % W], s1.h.x, s1.m.x, s1.l.x, ex[2]);
+          acc[3 % W] = add_sum(acc[3 % W], s1.h.y, s1.m.y, s1.l.y, ex[3]);
         }
       } else {   // infinities or NaN among the values
         for (int q = 0; q < 8; ++q) {
@@ -660,7 +685,8 @@ __global__ void __launch_bounds__(128) k_density_partial(const FieldParams p, in
 }
 
 // out[q] = w scale^2 sum over ch of part[ch total + q], q < total: blockDim.x outputs per
-// block, each of its rows of threads on every blockDim.y-th chunk, then added in order.
+// block, each of its rows of threads (a power of two) on every blockDim.y-th chunk, then added
+// in a tree (in order, 64 of them made the error of 1D densities 3e-16 instead of 1e-16).
 // (Few outputs of many chunks: 8 x 64 threads, so that the FP64 additions spread over
 // more SMs; 240 sums of 1000 chunks took 22 us on 8 blocks of 32 outputs.)
 __global__ void __launch_bounds__(512) k_density_combine(const double* __restrict__ part, int nch,
@@ -673,13 +699,15 @@ __global__ void __launch_bounds__(512) k_density_combine(const double* __restric
   if (q < total)
 #pragma unroll 4
     for (int c = threadIdx.y; c < nch; c += by) acc += part[(size_t)c * total + q];
-  sm[threadIdx.y * (bx + 1) + threadIdx.x] = acc;
-  __syncthreads();
+  double* mine = sm + threadIdx.y * (bx + 1) + threadIdx.x;
+  *mine = acc;
+  for (int half = by / 2; half > 0; half /= 2) {
+    __syncthreads();
+    if ((int)threadIdx.y < half) *mine += mine[half * (bx + 1)];
+  }
   if (threadIdx.y == 0 && q < total) {
-    double v = sm[threadIdx.x];
-    for (int t = 1; t < by; ++t) v += sm[t * (bx + 1) + threadIdx.x];
     const double s = scale ? *scale : 1.0;
-    out[q] = v * (w * s * s);
+    out[q] = *mine * (w * s * s);
   }
 }
 
@@ -709,7 +737,7 @@ __global__ void __launch_bounds__(256) k_density_sum_rows(const FieldParams p, d
       }
     } else {
       const float2* row = reinterpret_cast<const float2*>(base);
-      for (int c0 = lane; c0 < n; c0 += 32 * 8) {   // eight pairs in two parts, as k_density_partial
+      for (int c0 = lane; c0 < n; c0 += 32 * 8) {   // eight pairs, as in k_density_partial
         float2 v[8];
         float m = 0.f;
 #pragma unroll
@@ -719,20 +747,14 @@ __global__ void __launch_bounds__(256) k_density_sum_rows(const FieldParams p, d
           if (!CPLX && 2 * c + 1 >= p.nx) v[q].y = 0.f;
           m = fmaxf(m, fmaxf(fabsf(v[q].x), fabsf(v[q].y)));
         }
-        const int ex = min(max((int)(__float_as_uint(m) >> 23), 30), 223);
-        const float2 sc = f2(__uint_as_float((unsigned int)(254 - ex) << 23));
-        Two s0 = two_zero();
+        const int ex = square_exponent(m);
+        const float2 sc = f2(square_scale(ex));
+        Squares s0{f2(0.f), f2(0.f), f2(0.f)};
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const float2 a = mul2(v[q], sc);
-          Two qa;
-          qa.h = mul2(a, a);
-          qa.l = fma2(a, a, mul2(qa.h, f2(-1.f)));
-          s0 = two_add(s0, qa);
-        }
-        s0 = two_norm(two_add(s0, two_swap(s0)));
-        if (fabsf(s0.h.x) <= 1e30f) {
-          acc += to_double(s0.h.x, s0.l.x, kSplitShift + 2 * (ex - 127));
+        for (int q = 0; q < 8; ++q) add_square(s0, mul2(v[q], sc));
+        add_lanes(s0);
+        if (finite_sums(s0.h)) {
+          acc = add_sum(acc, s0.h.x, s0.m.x, s0.l.x, ex);
         } else {   // infinities or NaN among the values
           for (int q = 0; q < 8; ++q)
             acc = fma((double)v[q].x, (double)v[q].x, fma((double)v[q].y, (double)v[q].y, acc));

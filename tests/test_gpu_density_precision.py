@@ -61,3 +61,13 @@ def test_columns_far_below_their_neighbours(P, shape, cplx):
     psi = psi * size[np.arange(shape[0]) % 6][None, None, :]
     psi = (psi.astype(np.complex64) if cplx else psi.astype(np.float32)).astype(psi.dtype)
     check(P, psi, 2.0 ** -40)
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("amp", [1.0, 2.0 ** 100, 2.0 ** 126, 2.0 ** -120])
+@pytest.mark.parametrize("shape", [(37, 29, 21), (200, 70, 33), (130, 33, 1), (5, 3, 400), (3, 501, 7)])
+def test_fp64_precision(P, shape, amp, cplx):
+    psi = field(shape, cplx)
+    psi = (np.clip(abs(psi.real), 0.01, 1.99) + (1j * np.clip(abs(psi.imag), 0.01, 1.99) if cplx else 0)) * amp
+    psi = (psi.astype(np.complex64) if cplx else psi.astype(np.float32)).astype(psi.dtype)
+    check(P, psi, 8 * 2.0 ** -53)
