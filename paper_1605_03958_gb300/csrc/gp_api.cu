@@ -428,6 +428,8 @@ FieldParams field_params(gp_solver* s) {
   f.hy = s->prm.dy;
   f.hz = s->prm.nz == 1 ? 1.0 : s->prm.dz;   // 2D: cell area hx hy
   f.g = s->g;
+  const double w[3] = {s->prm.gamma, s->prm.nu, s->prm.lambda};
+  for (int a = 0; a < 3; ++a) f.v2[a] = 0.5 * w[a] * w[a];
   f.amax = s->line64 ? amax_words(s) : nullptr;
   return f;
 }

@@ -198,6 +198,9 @@ FieldParams slot_field(gp_pool* P, int slot) {
   f.hy = S.prm.dy;
   f.hz = S.prm.dz;
   f.g = S.g;
+  f.v2[0] = 0.5 * S.prm.gamma * S.prm.gamma;
+  f.v2[1] = 0.5 * S.prm.nu * S.prm.nu;
+  f.v2[2] = 0.5 * S.prm.lambda * S.prm.lambda;
   return f;
 }
 

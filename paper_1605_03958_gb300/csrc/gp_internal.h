@@ -209,6 +209,7 @@ struct FieldParams {
   int* status;
   const double* tab;     // FP64 tables: V_x[nx] V_y[ny] V_z[nz] x^2[nx] y^2[ny] z^2[nz]
   double hx, hy, hz, g;
+  double v2[3] = {};     // V_a(x) = v2[a] x^2
   int* amax = nullptr;   // FP64 solves: kAmaxNow receives the values written (import, Gaussian); else null
 };
 

@@ -159,33 +159,73 @@ __global__ void __launch_bounds__(kReduceThreads) k_observables(const FieldParam
 // The same sums with the arithmetic on the FP32 pipe (gp_split.cuh: FP64 operations and
 // conversions run at 1/64 of FP32's rate here, and k_observables spends 32-45 of them per
 // point: 590 us for 240 x 200 x 160 complex64 points, where reading the field takes 9 us).
-// FP32 values are taken as they are, FP64 ones as two FP32 parts (48 bits, rounded to
-// nearest, so the terms' errors are independent and average out over the field); squares
-// and sums are two-part (2^-48 per addition), one FP64 conversion per thread and sum.  The
-// weights are exact: x^2 = (2i - nx + 1)^2 h^2 / 4 with the integer part in FP32, and the
-// potential energy follows from the three weighted sums.  The pending factor is applied
+// FP32 values are taken as they are, FP64 ones as three FP32 parts, all 53 bits: their
+// differences are exact that way (from 48 bits the kinetic sum of a finely sampled field is off by
+// 2^-48 over the relative difference of neighbours).  Squares are two-part; a sum of them has
+// three parts, adds without error but for its third part's rounding, and moves to FP64 (in shared
+// memory) every two dozen terms.  With two-part sums the low part was rounded at every
+// addition, and because a sum of two squares is never 3 mod 4 in its last bits, ties went down
+// more often than up: sums 2e-16..5e-16 too small, fourth powers 1e-15.  The weights
+// are exact in x: (2i - nx + 1)^2 h^2 / 4 with the integer part in FP32; y and z weigh a row's
+// sum in FP64; the potential energy follows from the three.  The pending factor is applied
 // to the sums.  Fields whose largest value (times the factor) lies outside
 // [2^-16, 2^24], where sums of weighted fourth powers could leave FP32's range, and small grids (fewer than
 // 2^15 points, where k_observables takes no longer and there is less to average over) go
 // to k_observables; out[10] receives the largest |component| and out[11] the factor for the
 // host's check.
-// Measured (240 x 200 x 160, the whole call): complex64 736 -> 138 us, FP64 real 451 -> 112,
-// complex128 611 -> 170; the kernel (complex64, 110 us) is bound by its 216 instructions per
-// point, FP32 39 % of the pipe.  Error of the sums against quadruple precision at most a few
-// 1e-16 relative, as before (160 x 120 x 100 FP64: energy 1.3e-16, norm 2.6e-16).
+// Measured (240 x 200 x 160, the whole call): complex64 736 -> 187 us, FP32 real 124, FP64 real
+// 451 -> 159, complex128 611 -> 250; bound by its FP32 instructions.  Error against extended
+// precision as k_observables': at most 4 x 2^-53 relative, no lean to one side (two-part sums: 137
+// us and up to 17 x 2^-53).
 // A warp takes a row at a time, consecutive warps consecutive rows (y neighbours from L1),
 // the next 32 columns' loads in flight.
 constexpr int kObsTwoBlocks = 304;   // two resident blocks per SM
 
-template <class R, bool CPLX> struct PairLoad;   // columns (2c, 2c + 1), or (re, im) of column c
+// A value pair: columns (2c, 2c + 1), or (re, im) of column c.
+template <class R> struct PairValue;
+template <> struct PairValue<float> {
+  float2 v;
+  __device__ __forceinline__ float2 high() const { return v; }
+  __device__ __forceinline__ Two two() const { return two_scalar(v, f2(0.f)); }
+  __device__ __forceinline__ PairValue next(const PairValue& n) const { return {f2(v.y, n.v.x)}; }   // one column on
+  __device__ __forceinline__ Two minus(const PairValue& b) const {
+    Two d;
+    two_sum(v, mul2(b.v, f2(-1.f)), &d.h, &d.l);
+    return d;
+  }
+};
+template <> struct PairValue<double> {
+  Three v;
+  __device__ __forceinline__ float2 high() const { return v.h; }
+  __device__ __forceinline__ Two two() const {
+    const float2 h = add2(v.h, v.m);
+    return two_scalar(h, add2(sub2(v.m, sub2(h, v.h)), v.l));
+  }
+  __device__ __forceinline__ PairValue next(const PairValue& n) const {
+    PairValue r;
+    r.v.h = f2(v.h.y, n.v.h.x);
+    r.v.m = f2(v.m.y, n.v.m.x);
+    r.v.l = f2(v.l.y, n.v.l.x);
+    return r;
+  }
+  __device__ __forceinline__ Two minus(const PairValue& b) const {
+    float2 s, e, f;
+    two_sum(v.h, mul2(b.v.h, f2(-1.f)), &s, &e);
+    Two d;
+    two_sum(s, sub2(v.m, b.v.m), &d.h, &f);
+    d.l = add2(f, add2(sub2(v.l, b.v.l), e));
+    return d;
+  }
+};
+template <class R, bool CPLX> struct PairLoad;
 template <bool CPLX> struct PairLoad<float, CPLX> {
   using V = float2;
   static __device__ __forceinline__ V load(const void* row, int c, int nc) {   // zero from nc on
     return c < nc ? static_cast<const float2*>(row)[c] : f2(0.f);
   }
-  static __device__ __forceinline__ Two two(V v, int c, int nx) {
+  static __device__ __forceinline__ PairValue<float> value(V v, int c, int nx, int*) {
     if (!CPLX && 2 * c + 1 >= nx) v.y = 0.f;
-    return two_scalar(v, f2(0.f));
+    return {v};
   }
 };
 template <bool CPLX> struct PairLoad<double, CPLX> {
@@ -193,13 +233,31 @@ template <bool CPLX> struct PairLoad<double, CPLX> {
   static __device__ __forceinline__ V load(const void* row, int c, int nc) {
     return c < nc ? static_cast<const double2*>(row)[c] : make_double2(0.0, 0.0);
   }
-  static __device__ __forceinline__ Two two(V v, int c, int nx) {
+  static __device__ __forceinline__ PairValue<double> value(V v, int c, int nx, int* tmax) {
     if (!CPLX && 2 * c + 1 >= nx) v.y = 0.0;
-    int tmax = 0;
-    const Two t = split2(v.x, v.y, &tmax);
-    // out of range: an infinity, for the host's check
-    const float s = tmax >= kSplitTooBig ? __int_as_float(0x7f800000) : 0x1p-56f;
-    return two_scalar(mul2(t.h, f2(s)), mul2(t.l, f2(s)));
+    PairValue<double> r;
+    r.v = split3(v.x, v.y, tmax, kSplitOff1);
+    return r;
+  }
+};
+
+// A sum of two-part numbers in three parts, two lanes.
+struct SquareSum {
+  float2 h = make_float2(0.f, 0.f), l = h, m = h;
+  __device__ __forceinline__ void add(const Two& q) {
+    float2 f, g, k, t;
+    two_sum(h, q.h, &t, &f);
+    h = t;
+    two_sum(l, q.l, &t, &g);
+    two_sum(t, f, &l, &k);
+    m = add2(m, add2(g, k));
+  }
+  // lane x, or both lanes (NaN: infinities or NaN among the values)
+  __device__ __forceinline__ double total(bool both) const {
+    auto d = [](float x) { return to_double(x, 0.f, kSplitShift); };
+    double s = (d(h.x) + d(l.x)) + d(m.x);
+    if (both) s += (d(h.y) + d(l.y)) + d(m.y);
+    return fabsf(h.x) + fabsf(h.y) <= 1e30f ? s : (double)__int_as_float(0x7fc00000);
   }
 };
 
@@ -213,33 +271,46 @@ __global__ void __launch_bounds__(kReduceThreads, 2) k_observables_two(const Fie
   const int nrows = ny * nz;
   using L = PairLoad<R, CPLX>;
   constexpr bool LOW = sizeof(R) == 8;   // values have low parts
-  // v^2 without the square of the low part, which (never negative) would always round away:
-  // those are summed by themselves in `low`; renormalised, so that the sums' low parts stay
-  // small
-  auto square = [](const Two& v, float2* low) {
+  // v^2 = q.h + q.l + what `low` receives, which all sums take in FP64 at the end (rounded away,
+  // the square of the low part, never negative, would bias them).  full: nothing rounds but low
+  // itself; else q.l does, which is exact for a v without a low part.
+  auto square = [](const Two& v, float2* low, bool full) {
     Two q;
+    const float2 v2 = add2(v.h, v.h);
     q.h = mul2(v.h, v.h);
-    q.l = fma2(add2(v.h, v.h), v.l, fma2(v.h, v.h, mul2(q.h, f2(-1.f))));
+    const float2 res = fma2(v.h, v.h, mul2(q.h, f2(-1.f)));
     *low = fma2(v.l, v.l, *low);
-    return two_scalar(add2(q.h, q.l), sub2(q.l, sub2(add2(q.h, q.l), q.h)));
+    if (full) {
+      const float2 p = mul2(v2, v.l), pe = fma2(v2, v.l, mul2(p, f2(-1.f)));
+      float2 e;
+      two_sum(res, p, &q.l, &e);
+      *low = add2(*low, add2(e, pe));
+    } else {
+      q.l = fma2(v2, v.l, res);
+    }
+    return q;
   };
-  auto edge = [&](const Two& a, const Two& b, float2* low) {   // |a - b|^2
-    Two d;
-    float2 e;
-    const Two n = two_neg(b);
-    two_sum(a.h, n.h, &d.h, &e);
-    d.l = LOW ? add2(add2(a.l, n.l), e) : e;
-    return square(d, low);
-  };
+  auto edge = [&](const PairValue<R>& a, const PairValue<R>& b, float2* low) { return square(a.minus(b), low, LOW); };
   float2 lSX = f2(0.f), lS4 = f2(0.f), lX = f2(0.f), lY = f2(0.f), lZ = f2(0.f);
-  Two S = two_zero(), SX = two_zero(), SY = two_zero(), SZ = two_zero(), S4 = two_zero(), KX = two_zero(),
-      KY = two_zero(), KZ = two_zero();
+  float lS = 0.f, lSY = 0.f, lSZ = 0.f;
+  SquareSum SX, S4, KX, KY, KZ;
   float vmax = 0.f;
+  int tmax = 0;
+  __shared__ double sums[8][kReduceThreads];   // S, SX, SY, SZ, S4, KX, KY, KZ
+  auto drain = [&](int i, SquareSum& t, bool both) {
+    sums[i][threadIdx.x] += t.total(both);
+    t = SquareSum();
+  };
+#pragma unroll
+  for (int i = 0; i < 8; ++i) sums[i][threadIdx.x] = 0.0;
+  const double* Y2 = p.tab + 2 * nx + ny + nz;   // y^2, then z^2
+  const int often = max(1, 24 / ((nc + 31) / 32));   // rows between two drains
+  int due = often;
   const int step = gridDim.x * (kReduceThreads / 32);
   for (int r = blockIdx.x * (kReduceThreads / 32) + (threadIdx.x >> 5); r < nrows; r += step) {
     const int k = r / ny, j = r - k * ny;
     const unsigned char* row = field + (size_t)r * rowb;
-    Two SR = two_zero();
+    SquareSum SR;
     float2 lSR = f2(0.f);
     auto fetch = [&](int c, typename L::V (&b)[4]) {   // a point and its three neighbours
       b[0] = L::load(row, c, nc);
@@ -251,56 +322,92 @@ __global__ void __launch_bounds__(kReduceThreads, 2) k_observables_two(const Fie
     fetch(lane, cur);
     for (int c = lane; c < nc; c += 32) {
       fetch(c + 32, ahead);
-      const Two v = L::two(cur[0], c, nx), nxt = L::two(cur[1], c + 1, nx), wy = L::two(cur[2], c, nx),
-                wz = L::two(cur[3], c, nx);
+      const PairValue<R> at = L::value(cur[0], c, nx, &tmax), nxt = L::value(cur[1], c + 1, nx, &tmax),
+                         wy = L::value(cur[2], c, nx, &tmax), wz = L::value(cur[3], c, nx, &tmax);
+      const Two v = at.two();
 #pragma unroll
       for (int q = 0; q < 4; ++q) cur[q] = ahead[q];
-      const Two wx = CPLX ? nxt : two_scalar(f2(v.h.y, nxt.h.x), f2(v.l.y, nxt.l.x));
+      const PairValue<R> wx = CPLX ? nxt : at.next(nxt);
       vmax = fmaxf(vmax, fmaxf(fabsf(v.h.x), fabsf(v.h.y)));
       float2 ll = f2(0.f);
-      const Two q = square(v, &ll);
-      SR = two_add(SR, q);
+      const Two q = square(v, &ll, LOW);
+      SR.add(q);
       lSR = add2(lSR, ll);
       // (2i - nx + 1)^2 below 2^22: exact in FP32
       const float w0 = (float)(2 * (CPLX ? c : 2 * c) - nx + 1), w1 = CPLX ? w0 : w0 + 2.f;
       const float2 wc = f2(w0 * w0, w1 * w1);
-      SX = two_add(SX, two_mul(two_scalar(wc, f2(0.f)), q));
-      const Two d = CPLX ? two_add(q, two_swap(q)) : q;
-      S4 = two_add(S4, square(d, &lS4));
+      Two qx;
+      qx.h = mul2(wc, q.h);
+      qx.l = fma2(wc, q.l, fma2(wc, q.h, mul2(qx.h, f2(-1.f))));
+      SX.add(qx);
+      Two d = q;
+      float2 rest = f2(0.f);   // of d
+      if (CPLX) {
+        const Two o = two_swap(q);
+        float2 e, f, l, g;
+        two_sum(q.h, o.h, &d.h, &e);
+        two_sum(q.l, o.l, &l, &f);
+        two_sum(l, e, &d.l, &g);
+        rest = add2(f, g);
+      }
+      S4.add(square(d, &lS4, true));
+      if (CPLX) lS4 = fma2(add2(d.h, d.h), rest, lS4);
       if (LOW) {   // the squares of the values' low parts in the weighted and fourth-power sums
         lSX = fma2(wc, ll, lSX);
         lS4 = fma2(add2(d.h, d.h), CPLX ? add2(ll, f2(ll.y, ll.x)) : ll, lS4);
       }
-      KX = two_add(KX, edge(wx, v, &lX));
-      KY = two_add(KY, edge(wy, v, &lY));
-      KZ = two_add(KZ, edge(wz, v, &lZ));
+      KX.add(edge(wx, at, &lX));
+      KY.add(edge(wy, at, &lY));
+      KZ.add(edge(wz, at, &lZ));
       if (c == 0) {   // the ghost edge at i = 0
         const float2 m = f2(1.f, CPLX ? 1.f : 0.f);
-        KX = two_add(KX, two_scalar(mul2(q.h, m), mul2(q.l, m)));
+        KX.add(two_scalar(mul2(q.h, m), mul2(q.l, m)));
+        if (LOW) lX = fma2(m, ll, lX);
       }
-      if (j == 0) KY = two_add(KY, q);
-      if (k == 0) KZ = two_add(KZ, q);
+      if (j == 0) {
+        KY.add(q);
+        if (LOW) lY = add2(lY, ll);
+      }
+      if (k == 0) {
+        KZ.add(q);
+        if (LOW) lZ = add2(lZ, ll);
+      }
     }
-    if (LOW) SR = two_add(SR, two_scalar(lSR, f2(0.f)));
-    S = two_add(S, SR);
-    const float wj = (float)(2 * j - ny + 1), wk = (float)(2 * k - nz + 1);
-    SY = two_add(SY, two_mul(two_scalar(f2(wj * wj), f2(0.f)), SR));
-    SZ = two_add(SZ, two_mul(two_scalar(f2(wk * wk), f2(0.f)), SR));
+    {
+      const double sr = SR.total(true), y2 = Y2[j], z2 = Y2[ny + k];
+      sums[0][threadIdx.x] += sr;
+      sums[2][threadIdx.x] = fma(y2, sr, sums[2][threadIdx.x]);
+      sums[3][threadIdx.x] = fma(z2, sr, sums[3][threadIdx.x]);
+      if (LOW) {
+        const float lr = lSR.x + lSR.y;
+        lS += lr;
+        lSY = fmaf((float)y2, lr, lSY);
+        lSZ = fmaf((float)z2, lr, lSZ);
+      }
+    }
+    if (--due > 0 && r + step < nrows) continue;
+    due = often;
+    drain(1, SX, true);
+    drain(4, S4, !CPLX);
+    drain(5, KX, true);
+    drain(6, KY, true);
+    drain(7, KZ, true);
   }
-  auto total = [](const Two& t, bool both) {
-    const Two n = two_norm(t);
-    if (!(fabsf(n.h.x) + fabsf(n.h.y) <= 1e30f)) return (double)__int_as_float(0x7fc00000);   // NaN among the values
-    const double a = to_double(n.h.x, n.l.x, kSplitShift);
-    return both ? a + to_double(n.h.y, n.l.y, kSplitShift) : a;
-  };
-  auto with = [](const Two& t, float2 low) { return two_add(t, two_scalar(low, f2(0.f))); };
-  SX = with(SX, lSX);
-  S4 = with(S4, lS4);
-  KX = with(KX, lX);
-  KY = with(KY, lY);
-  KZ = with(KZ, lZ);
-  double acc[8] = {total(S, true),        total(SX, true), total(SY, true), total(SZ, true),
-                   total(S4, !CPLX), total(KX, true), total(KY, true), total(KZ, true)};
+  if (LOW && tmax >= kSplitTooBig) vmax = __int_as_float(0x7f800000);   // out of FP32's range, for the host's check
+  double acc[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) acc[i] = sums[i][threadIdx.x];
+  auto both = [](float2 l) { return (double)l.x + (double)l.y; };
+  acc[4] += CPLX ? (double)lS4.x : both(lS4);
+  acc[5] += both(lX);
+  acc[6] += both(lY);
+  acc[7] += both(lZ);
+  if (LOW) {
+    acc[0] += (double)lS;
+    acc[1] += both(lSX);
+    acc[2] += (double)lSY;
+    acc[3] += (double)lSZ;
+  }
   const unsigned int wmax = __reduce_max_sync(0xffffffffu, __float_as_uint(vmax));
   __shared__ unsigned int bmax;
   if (threadIdx.x == 0) bmax = 0u;
@@ -318,19 +425,20 @@ __global__ void __launch_bounds__(kReduceThreads, 2) k_observables_two(const Fie
   if (lane == 0) atomicMax(&bmax, m);
   __syncthreads();
   if (threadIdx.x == 0) {
-    const double s = *p.scale, s2 = s * s, dV = p.hx * p.hy * p.hz;
-    const double* Vx = p.tab;
-    const double* X2 = Vx + nx + ny + nz;
-    const double sum = tot[0] * s2, norm = sum * dV;
-    const double sx = tot[1] * s2 * (0.25 * p.hx * p.hx), sy = tot[2] * s2 * (0.25 * p.hy * p.hy);
-    const double sz = nz == 1 ? 0.0 : tot[3] * s2 * (0.25 * p.hz * p.hz);
-    // V_a(x) = (w_a^2 / 2) x^2: the tables' ratio at the first point (nonzero there)
-    const double epot = (sx * (Vx[0] / X2[0]) + sy * (Vx[nx] / X2[nx]) +
-                         (nz == 1 ? 0.0 : sz * (Vx[nx + ny] / X2[nx + ny]))) * dV;
-    const double eint = 0.5 * p.g * (tot[4] * s2 * s2) * dV;
-    const double ekin = 0.5 * dV * s2 * (tot[5] / (p.hx * p.hx) + tot[6] / (p.hy * p.hy) +
-                                         (nz == 1 ? 0.0 : tot[7] / (p.hz * p.hz)));
-    const double x2 = sx * dV / norm, y2 = sy * dV / norm, z2 = sz * dV / norm;
+    // (products of constants in an order, and with a remainder, that leave no rounding error that
+    // would be the same for every field)
+    const double s = *p.scale, s2 = s * s;
+    const double area = p.hx * p.hy, dV = area * p.hz;
+    const double dVl = fma(area, p.hz, -dV) + fma(p.hx, p.hy, -area) * p.hz;
+    auto integral = [&](double x) { return fma(x, dVl, x * dV); };
+    const double sum = tot[0] * s2, norm = integral(sum);
+    const double sx = tot[1] * s2 * 0.25 * p.hx * p.hx, sy = tot[2] * s2;
+    const double sz = nz == 1 ? 0.0 : tot[3] * s2;
+    const double epot = integral(sx * p.v2[0] + sy * p.v2[1] + sz * p.v2[2]);
+    const double eint = integral(tot[4] * s2 * s2 * (0.5 * p.g));
+    const double ekin = integral(0.5 * s2 * (tot[5] / p.hx / p.hx + tot[6] / p.hy / p.hy +
+                                             (nz == 1 ? 0.0 : tot[7] / p.hz / p.hz)));
+    const double x2 = sx / sum, y2 = sy / sum, z2 = sz / sum;
     double* o = p.out;
     o[0] = norm;
     o[1] = ekin + epot + 2.0 * eint;

@@ -36,6 +36,7 @@ namespace gpk {
 constexpr int kSplitShift = 56;
 // FP64 exponent field minus kSplitOff is the FP32 exponent field of v 2^kSplitShift
 constexpr int kSplitOff = (1023 - 127 - kSplitShift) << 20;
+constexpr int kSplitOff1 = (1023 - 127) << 20;   // of v itself
 // split3's tmax from which the value is too large (FP32 exponent field 250)
 constexpr int kSplitTooBig = 250 << 20;
 
@@ -337,17 +338,18 @@ GP_HD Two two_square_up(const Two& q) {
 // Two FP64 values times 2^kSplitShift as h + m + l exactly: h the leading 21 bits, m and
 // l the next 16 and 16.  Sums of a few m (or l) of neighbouring values are exact (16-bit
 // integers times nearby powers of two).  *tmax receives the larger of itself and the
-// values' exponent fields (kSplitTooBig: out of range or non-finite).
+// values' exponent fields (kSplitTooBig: out of range or non-finite).  With off = kSplitOff1 the
+// values themselves (FP32's range and no more).
 struct Three {
   float2 h, m, l;
 };
-GP_HD Three split3(double a, double b, int* tmax) {
+GP_HD Three split3(double a, double b, int* tmax, int off = kSplitOff) {
   uint32_t h[2], o[2];
   words(a, &h[0], &o[0]);
   words(b, &h[1], &o[1]);
   float hf[2], p[2], mf[2], lf[2];
   for (int q = 0; q < 2; ++q) {
-    const int t = addmax0((int)(h[q] & 0x7fffffffu), -kSplitOff);
+    const int t = addmax0((int)(h[q] & 0x7fffffffu), -off);
     *tmax = imax(*tmax, t);
     const uint32_t w = ((uint32_t)t << 3) | (h[q] & 0x80000000u);
     hf[q] = bits_f(w);
