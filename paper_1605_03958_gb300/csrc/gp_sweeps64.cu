@@ -990,10 +990,13 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
     struct IO {
       float4* slot;
       const double* row[2];   // v' of the thread's row(s) in the field
-      int TS, j0, nx;
+      int TS, j0, nx, pitch;
       bool on;
+      long long first, nall;   // bounds checks: first vector of row[0], the field's vectors
+      int* status;
       __device__ double2 rd(int j) const {
         if (!on || j < 0 || j >= nx) return make_double2(0.0, 0.0);
+        if (!GP_IN(first + (!CPLX && row[1] ? pitch : 0) + (CPLX ? j : j / 2), nall, status)) return make_double2(0.0, 0.0);
         if constexpr (CPLX) return reinterpret_cast<const double2*>(row[0])[j];
         return make_double2(row[0][j], row[1] ? row[1][j] : 0.0);
       }
@@ -1005,6 +1008,10 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
     io.TS = TS;
     io.j0 = j0;
     io.nx = nx;
+    io.pitch = P;
+    io.first = at0 + (long long)(xl * RPV) * P;
+    io.nall = nall;
+    io.status = p.status;
     io.row[0] = reinterpret_cast<const double*>(field + (size_t)(xl * RPV) * P);
     io.row[1] = !CPLX && xl * RPV + 1 < rows ? reinterpret_cast<const double*>(field + (size_t)(xl * RPV + 1) * P)
                                              : nullptr;
