@@ -514,7 +514,7 @@ void fill_sweep_params(gp_solver* s) {
         q.inc_ex = coef + s->L.ex_off[m];
         q.inc_amax = amax_words(s);
         if (!gpk::inc64_setup(a, &q, m == 0 ? std::complex<double>(beta, 0.0)
-                                             : std::complex<double>(0.0, beta), m == 1) ||
+                                             : std::complex<double>(0.0, beta), m == 1, s->nsm) ||
             (a > 0 && gpk::inc64_blocks(a, q, m == 1) > (long long)s->L.npartials))
           q.inc_x = 0;
         q.plane_norm = q.inc_x && p.nz == 1 && a == 1 && m == 0 ? 1 : 0;

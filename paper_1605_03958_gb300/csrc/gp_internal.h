@@ -102,7 +102,7 @@ struct SweepParams {
   // FP64 increment sweeps (gp_sweeps64.cu): decay factor rho of the CN solve's two
   // one-sided recursions, rho + 1/rho = (1+2a)/a, in FP64 (re, im) and as the FP32 pairs
   // (re hi, re lo, im hi, im lo); 16-byte vectors per block row and segments per line
-  int inc_x, inc_seg;    // inc_x = 0: not used
+  int inc_x, inc_seg, inc_threads;   // inc_x = 0: not used; threads per block
   double rho[2];
   float rho_f[4];
   float inc_rough;       // rms(v)^2 / rms(s)^2 up to which a block is rough, s the second difference
@@ -281,8 +281,8 @@ long long sweep64_blocks(int axis, int nx, int ny, int nz);
 cudaError_t launch_sweep64(int axis, const SweepParams& p, bool complex_field, cudaStream_t st);
 // FP64 increment form of the sweeps: whether a line of n points with CN parameter
 // a (real: imaginary time, imaginary: real time) qualifies; fills p's inc_* and rho
-// fields (p.n, p.nx, p.ny, p.nz set); blocks of the launch, and the launch.
-bool inc64_setup(int axis, SweepParams* p, std::complex<double> a, bool complex_field);
+// fields (p.n, p.nx, p.ny, p.nz set; nsm: the device's SMs); blocks of the launch, and the launch.
+bool inc64_setup(int axis, SweepParams* p, std::complex<double> a, bool complex_field, int nsm);
 long long inc64_blocks(int axis, const SweepParams& p, bool complex_field);
 cudaError_t launch_inc64(int axis, const SweepParams& p, bool complex_field, cudaStream_t st);
 // Resident warps per SM of the streaming y / z kernel (occupancy calculator).

@@ -185,7 +185,6 @@ constexpr int kObsTwoBlocks = 304;   // two resident blocks per SM
 template <class R> struct PairValue;
 template <> struct PairValue<float> {
   float2 v;
-  __device__ __forceinline__ float2 high() const { return v; }
   __device__ __forceinline__ Two two() const { return two_scalar(v, f2(0.f)); }
   __device__ __forceinline__ PairValue next(const PairValue& n) const { return {f2(v.y, n.v.x)}; }   // one column on
   __device__ __forceinline__ Two minus(const PairValue& b) const {
@@ -196,7 +195,6 @@ template <> struct PairValue<float> {
 };
 template <> struct PairValue<double> {
   Three v;
-  __device__ __forceinline__ float2 high() const { return v.h; }
   __device__ __forceinline__ Two two() const {
     const float2 h = add2(v.h, v.m);
     return two_scalar(h, add2(sub2(v.m, sub2(h, v.h)), v.l));

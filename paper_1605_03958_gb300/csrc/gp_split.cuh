@@ -327,14 +327,6 @@ GP_HD Two two_cis_neg_m1_small(const Two& y) {
   const float m = -y.h.y, ml = -y.l.y + y.h.y * re * (1.f / 6.f);
   return two_scalar(f2(c, m), f2(cl, ml));
 }
-// exp(-2 y) - 1 from q = exp(-y) - 1
-GP_HD Two two_square_up(const Two& q) {
-  Two d;
-  d.h = add2(q.h, q.h);
-  d.l = add2(q.l, q.l);
-  return two_add(d, two_mul(q, q));
-}
-
 // Two FP64 values times 2^kSplitShift as h + m + l exactly: h the leading 21 bits, m and
 // l the next 16 and 16.  Sums of a few m (or l) of neighbouring values are exact (16-bit
 // integers times nearby powers of two).  *tmax receives the larger of itself and the

@@ -461,7 +461,6 @@ constexpr int kIncG = 4;         // values of v read ahead in the backward pass
 constexpr int kIncH = 12;        // terms of a carry
 constexpr int kIncNear = 6;      // of those, the near ones in two-part arithmetic
 constexpr int kIncThreads = 256; // most threads per block
-constexpr int kIncSms = 152;     // SMs of a GB300
 constexpr double kIncRough = 128.0;  // a block is rough from rms(v) / rms(s) = kIncRough |a|
 
 // Fields of that size and less are not for FP32's exponent range (gp_split.cuh): increments
@@ -1096,7 +1095,7 @@ cudaError_t launch_sweep64(int axis, const SweepParams& p, bool complex_field, c
 // a <= 1/32 (rho^12 < 2^-60).  Positions per block: enough for about 256 threads on short
 // lines, fewer on long ones so that a block keeps to kIncThreads; whole tiles of nearly
 // equal width.
-bool inc64_setup(int axis, SweepParams* p, std::complex<double> a, bool complex_field) {
+bool inc64_setup(int axis, SweepParams* p, std::complex<double> a, bool complex_field, int nsm) {
   p->inc_x = 0;
   if (p->n < 16 || std::abs(a) > 1.0 / 32) return false;
   // block rows: 16-byte vectors along x (y, z sweeps) or pairs of rows / rows (x sweep)
@@ -1110,9 +1109,14 @@ bool inc64_setup(int axis, SweepParams* p, std::complex<double> a, bool complex_
   // more rows a block has, and a block more than its neighbours an SM's whole share: 128 x 96 x 64
   // 192 blocks 41 us, 280 33; 64 x 48 x 32 24 blocks 18.5 us, 128 14.6, complex 48 blocks 20.5,
   // 140 16.6; 300 x 256 plane 22 blocks 21 us, 128 14.8)
-  if (axis == 0) tiles = (tiles + kIncSms - 1) / kIncSms * kIncSms;
+  if (axis == 0) tiles = (tiles + nsm - 1) / nsm * nsm;
   p->inc_seg = nseg;
   p->inc_x = (nvec + tiles - 1) / tiles;
+  p->inc_threads = (p->inc_x * nseg + 31) / 32 * 32;
+  // x, grids of at most two blocks per SM: more threads than segments share the passes along the
+  // rows (64 x 48 x 32, then 24 blocks: x 22.5 -> 19.3 us, 101 x 77 x 53 complex step 75 -> 58 us;
+  // larger grids would lose resident blocks)
+  if (axis == 0 && (nvec + p->inc_x - 1) / p->inc_x <= 2 * nsm) p->inc_threads = kIncThreads;
   p->inc_rough = (float)(kIncRough * kIncRough * std::norm(a));
   const std::complex<double> r = 2.0 * a / (1.0 + 2.0 * a + std::sqrt(1.0 + 4.0 * a));
   const double part[2] = {r.real(), r.imag()};
@@ -1167,13 +1171,9 @@ cudaError_t launch_inc64(int axis, const SweepParams& p, bool complex_field, cud
   cfg.numAttrs = 1;
   cfg.stream = st;
   cfg.gridDim = dim3((unsigned)inc64_blocks(axis, p, complex_field));
-  cfg.blockDim = dim3((unsigned)((p.inc_x * p.inc_seg + 31) / 32 * 32));
+  cfg.blockDim = dim3((unsigned)p.inc_threads);
   cfg.dynamicSmemBytes = (size_t)(kIncL + 2) * cfg.blockDim.x * sizeof(float4);
   if (axis == 0) {
-    // grids of at most two blocks per SM: more threads than segments share the passes along
-    // the rows (64 x 48 x 32, then 24 blocks: x 22.5 -> 19.3 us, 101 x 77 x 53 complex step 75 -> 58 us; larger
-    // grids would lose resident blocks)
-    if (cfg.gridDim.x <= 304) cfg.blockDim.x = kIncThreads;
     cfg.dynamicSmemBytes = inc64_x_smem(cfg.blockDim.x, p.inc_x);
     // high word of the |v| below which |y| < 2^-56 (complex: each part), the folded factor
     // being at most 1.0625
