@@ -263,23 +263,28 @@ GP_HD Two two_const_fma(float2 ch, float2 cl, const Two& y, float2 a) {
   p.l = fma2(y.l, a, fma2(y.h, a, mul2(p.h, f2(-1.f))));
   return two_add(two_scalar(ch, cl), p);
 }
-// (exp(-y) - 1 + y) / y^2 for |y| <= 1/16 (Taylor; the terms of exp from y^5 on, below 2^-27,
-// in FP32)
-GP_HD Two two_exp_series(const Two& y) {
+// (exp(-y) - 1 + y) / y^2 (Taylor; FP32 from the y^5 term of exp on, in the long form from y^6:
+// an error of 2^-32 y^5, 2^-35 y^6 of exp, which the sizes of y it is taken for keep below 2^-56)
+template <bool LONG> GP_HD Two two_exp_series(const Two& y) {
   const float2 y1 = y.h;
   float2 a = fma2(y1, f2(1.f / 40320.f), f2(-1.f / 5040.f));
   a = fma2(y1, a, f2(1.f / 720.f));
-  a = fma2(y1, a, f2(-1.f / 120.f));
-  // 1/24, 1/6 as an FP32 pair
-  Two w = two_const_fma(f2(1.f / 24.f), f2((float)(1.0 / 24.0 - (double)(1.f / 24.f))), y, a);
+  Two w;   // 1/24, 1/6 and, long, 1/120 as an FP32 pair
+  if constexpr (LONG) {
+    w = two_const_fma(f2(-1.f / 120.f), f2((float)(-(1.0 / 120.0 - (double)(1.f / 120.f)))), y, a);
+    w = two_add(two_scalar(f2(1.f / 24.f), f2((float)(1.0 / 24.0 - (double)(1.f / 24.f)))), two_mul(y, w));
+  } else {
+    a = fma2(y1, a, f2(-1.f / 120.f));
+    w = two_const_fma(f2(1.f / 24.f), f2((float)(1.0 / 24.0 - (double)(1.f / 24.f))), y, a);
+  }
   w = two_add(two_scalar(f2(-1.f / 6.f), f2((float)(-(1.0 / 6.0 - (double)(1.f / 6.f))))), two_mul(y, w));
   return two_add(two_scalar(f2(0.5f), f2(0.f)), two_mul(y, w));
 }
-// exp(-y) - 1, and the same without its leading term, exp(-y) - 1 + y
+// exp(-y) - 1 for |y| <= 1/64, and the same without its leading term, exp(-y) - 1 + y, for |y| <= 1/16
 GP_HD Two two_expm1_neg(const Two& y) {
-  return two_mul(y, two_add(two_scalar(f2(-1.f), f2(0.f)), two_mul(y, two_exp_series(y))));
+  return two_mul(y, two_add(two_scalar(f2(-1.f), f2(0.f)), two_mul(y, two_exp_series<false>(y))));
 }
-GP_HD Two two_expm1_neg_rest(const Two& y) { return two_mul(y, two_mul(y, two_exp_series(y))); }
+GP_HD Two two_expm1_neg_rest(const Two& y) { return two_mul(y, two_mul(y, two_exp_series<true>(y))); }
 // exp(-y) - 1 for |y| <= 2^-9: y^3 and higher terms (below 2^-29) in FP32
 GP_HD Two two_expm1_neg_small(const Two& y) {
   const float2 y1 = y.h, y2 = mul2(y1, y1);

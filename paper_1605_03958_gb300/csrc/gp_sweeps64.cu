@@ -726,11 +726,12 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_inc64(const __grid_consta
 // two-part / FP64 products (1e-16), at |E| = 1e-3, 1/64, 0.1, 0.28: real 0.6 / 0.9, 0.8 / 0.9, 2.7 /
 // 1.0, 6.6 / 1.0, complex 0.6 / 1.1, 1.0 / 1.1, 5.0 / 1.1, 17 / 1.1; at y = 1/128, 0.02, 0.1: 0.7 /
 // 1.0, 1.2 / 1.1, 8.6 / 1.1 and (1/256) 0.7 / 1.0, 1.3 / 1.0, 5.4 / 1.2.  So
-//   |y| from kIncY to 1/16: q's leading term (-y, -i y) in FP64, four operations per real
+//   |y| from kIncY to kIncLead: q's leading term (-y, -i y) in FP64, four operations per real
 //     value and seven per complex one, the rest of e as before;
-//   |E| > kIncE: the substep in FP64, except for |E| up to kIncBigE where the value is so small
-//     against the field's largest that its error stays below 2^-10 of such an |E|'s there;
-//   |y| > 1/16, values out of range, a tiny field: in FP64,
+//   |E| from kIncE to kIncBigE: E in FP64 too, nine and eighteen operations, unless the value is so
+//     small against the field's largest that two parts' error stays below 2^-10 of such an |E|'s there;
+//   |y| > kIncLead, |E| > kIncBigE, values out of range, a tiny field: products in FP64 (they round the
+//     factors' product alike at every step: an error that grows with the steps),
 // each for a warp as a whole.
 // Measured at 240 x 200 x 160 with the solve: 284 us (k_sweep_x64 at its shortest
 // polynomial; 620 us where the density calls for the longer one) -> 92 us, complex 686
@@ -744,6 +745,7 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_inc64(const __grid_consta
 constexpr float kIncBigE = 0.25f;
 constexpr float kIncE = 1.f / 64;
 template <bool CPLX> constexpr float kIncY = CPLX ? 1.f / 256 : 1.f / 128;
+constexpr float kIncLead = 1.f / 16;
 
 // v' in FP64 (f: the folded factor times the trap factors; real, complex)
 __device__ __forceinline__ double pointwise64(double v, double f, double cy) {
@@ -776,24 +778,36 @@ __device__ __forceinline__ double2 pointwise64(double2 v, double2 f, double cy) 
   return cmul(cmul(v, f), make_double2(cs, -sn));
 }
 
-// The real pair's or complex value's v' with y's leading term in FP64 (|y| <= 1/16); e: E, V: v
-// in two parts, cyc: cy.
-template <bool CPLX> __device__ __forceinline__ double2 pointwise_lead(double2 v, Two e, const Two& V, const Coef& cyc, double cy) {
-  const Two h = two_scalar(mul2(V.h, f2(0x1p-56f)), mul2(V.l, f2(0x1p-56f)));
-  Two d = two_mul(h, h);
-  if (CPLX) d = two_add(d, two_swap(d));
-  const Two y = prod_two(two_mul(cyc, d));
-  const Two rest = CPLX ? two_cis_neg_rest(y) : two_expm1_neg_rest(y);
-  const Two q = two_add(rest, CPLX ? two_scalar(f2(0.f, -y.h.y), f2(0.f, -y.l.y)) : two_neg(y));
-  e = two_add(two_add(e, rest), CPLX ? two_cmul(e, q) : two_mul(e, q));
-  const Two c = two_norm(CPLX ? two_cmul(V, e) : e);
+// The real pair's or complex value's v' with the leading terms in FP64: y's (|y| <= kIncLead), and if
+// `wide` E's, from the column's factor(s) less 1 (ca, cb; complex: ca) and the row's (er), which loses
+// nothing to the factors' product; dense: y is not nothing; e: E, cyc: cy, V: v in two parts.
+template <bool CPLX>
+__device__ __forceinline__ double2 pointwise_lead(double2 v, Two e, const Two& V, const Coef& cyc, double cy, bool dense,
+                                                  bool wide, double2 ca, double2 er) {
+  Two rest = two_zero();
+  if (dense) {
+    const Two h = two_scalar(mul2(V.h, f2(0x1p-56f)), mul2(V.l, f2(0x1p-56f)));
+    Two d = two_mul(h, h);
+    if (CPLX) d = two_add(d, two_swap(d));
+    const Two y = prod_two(two_mul(cyc, d));
+    rest = CPLX ? two_cis_neg_rest(y) : two_expm1_neg_rest(y);
+    const Two q = two_add(rest, CPLX ? two_scalar(f2(0.f, -y.h.y), f2(0.f, -y.l.y)) : two_neg(y));
+    rest = two_add(rest, CPLX ? two_cmul(e, q) : two_mul(e, q));
+  }
+  if (!wide) rest = two_add(e, rest);
+  const Two c = two_norm(CPLX ? two_cmul(V, rest) : rest);
   const int k = CPLX ? 0 : kSplitShift;
   const double2 w = make_double2(to_double(c.h.x, c.l.x, k), to_double(c.h.y, c.l.y, k));
+  double2 E = make_double2(0.0, 0.0);
   if constexpr (CPLX) {
     const double th = cy * fma(v.x, v.x, v.y * v.y);
-    return make_double2(v.x + fma(th, v.y, w.x), v.y + fma(-th, v.x, w.y));
+    if (!wide) return make_double2(v.x + fma(th, v.y, w.x), v.y + fma(-th, v.x, w.y));
+    E = cfma(ca, er, make_double2(ca.x + er.x, ca.y + er.y));
+    const double2 dv = cfma(v, make_double2(E.x, E.y - th), w);
+    return make_double2(v.x + dv.x, v.y + dv.y);
   } else {
-    return make_double2(fma(v.x, fma(-cy * v.x, v.x, w.x), v.x), fma(v.y, fma(-cy * v.y, v.y, w.y), v.y));
+    if (wide) E = make_double2(fma(ca.x, er.x, ca.x + er.x), fma(ca.y, er.x, ca.y + er.x));
+    return make_double2(fma(v.x, E.x + fma(-cy * v.x, v.x, w.x), v.x), fma(v.y, E.y + fma(-cy * v.y, v.y, w.y), v.y));
   }
 }
 
@@ -859,7 +873,8 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
     }
   }
   __syncthreads();
-  const Coef cyc = coef_pair(f2((float)cy), f2((float)(cy - (double)(float)cy)));
+  const double cyp = pw ? cy : 0.0;
+  const Coef cyc = coef_pair(f2((float)cyp), f2((float)(cyp - (double)(float)cyp)));
   int vmax = 0;
   // In the two passes along the rows a thread keeps to one vector position (column) per
   // chunk of `per` positions and walks down the tile, `grp` rows at a time.  Column c of
@@ -945,25 +960,54 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
             v.x = fma(v.x, to_double(c.h.x, c.l.x, kSplitShift), v.x);
             v.y = fma(v.y, to_double(c.h.y, c.l.y, kSplitShift), v.y);
           }
-        } else if (__all_sync(0xffffffffu, (ok && ym <= 0.0625f) || !live)) {
-          v = pointwise_lead<CPLX>(v, factor(rc), V, cyc, cy);
-        } else if (live) {
-          const double c2 = pw ? cy : 0.0;
-          // |y| < 2^-56: the factor alone (the far field, where |E| is large and v small: two
-          // to ten FP64 operations instead of ten to thirty; 240 x 200 x 160 at h = 0.2, where
-          // that is most of the grid: x 237 -> 119 us, complex 453 -> 264)
-          const bool quiet = !pw || vm < p.inc_quiet;
-          if constexpr (!CPLX) {
-            const double fr = pw ? s * static_cast<const double*>(p.band_fyz)[r0 + r] : s;
-            const double* fx = static_cast<const double*>(p.band_fx);
-            const double f0 = pw ? fr * fx[2 * cv] : fr, f1 = pw ? fr * fx[2 * cv + 1] : fr;
-            v.x = quiet ? v.x * f0 : pointwise64(v.x, f0, c2);
-            v.y = quiet ? v.y * f1 : pointwise64(v.y, f1, c2);
-          } else {
-            const double2 rf = pw ? static_cast<const double2*>(p.band_fyz)[r0 + r] : make_double2(1.0, 0.0);
-            const double2 f = pw ? static_cast<const double2*>(p.band_fx)[cv] : make_double2(1.0, 0.0);
-            const double2 f0 = cmul(make_double2(s * f.x, s * f.y), rf);
-            v = quiet ? cmul(v, f0) : pointwise64(v, f0, c2);
+        } else {
+          int big = 0;
+          const Two W = split2(v.x, v.y, &big);
+          const bool wide = !__all_sync(0xffffffffu, ok || !live);
+          const bool fit = !tiny && em <= kIncBigE && ym <= kIncLead && big < kSplitTooBig;
+          if (__all_sync(0xffffffffu, fit || !live)) {
+            double2 ca = make_double2(0.0, 0.0), er = ca;
+            if (wide && live) {
+              // the column's factor less 1: small, from its two parts; else the FP64 factor's is closer
+              auto sum = [](float a, float b) { return to_double(a, 0.f, kSplitShift) + to_double(b, 0.f, kSplitShift); };
+              const bool parts = em <= 0.0625f;
+              if (pw) {
+                if (parts) {
+                  ca = make_double2(sum(ext.x, ext.z), sum(ext.y, ext.w));
+                } else if constexpr (CPLX) {
+                  ca = static_cast<const double2*>(p.band_fx)[cv];
+                  ca.x -= 1.0;
+                } else {
+                  const double* fx = static_cast<const double*>(p.band_fx) + 2 * cv;
+                  ca = make_double2(fx[0] - 1.0, fx[1] - 1.0);
+                }
+              }
+              if constexpr (CPLX) {
+                const double2 rf = pw ? static_cast<const double2*>(p.band_fyz)[r0 + r] : make_double2(1.0, 0.0);
+                er = make_double2(fma(rf.x, s, -1.0), rf.y * s);
+              } else {
+                er.x = fma(pw ? static_cast<const double*>(p.band_fyz)[r0 + r] : 1.0, s, -1.0);
+              }
+            }
+            const bool dense = pw && !__all_sync(0xffffffffu, vm < p.inc_quiet);
+            v = pointwise_lead<CPLX>(v, factor(rc), W, cyc, dense ? cyp : 0.0, dense, wide, ca, er);
+          } else if (live) {
+            // |y| < 2^-56: the factor alone (the far field, where |E| is large and v small: two
+            // to ten FP64 operations instead of ten to thirty; 240 x 200 x 160 at h = 0.2, where
+            // that is most of the grid: x 237 -> 119 us, complex 453 -> 264)
+            const bool quiet = !pw || vm < p.inc_quiet;
+            if constexpr (!CPLX) {
+              const double fr = pw ? s * static_cast<const double*>(p.band_fyz)[r0 + r] : s;
+              const double* fx = static_cast<const double*>(p.band_fx);
+              const double f0 = pw ? fr * fx[2 * cv] : fr, f1 = pw ? fr * fx[2 * cv + 1] : fr;
+              v.x = quiet ? v.x * f0 : pointwise64(v.x, f0, cyp);
+              v.y = quiet ? v.y * f1 : pointwise64(v.y, f1, cyp);
+            } else {
+              const double2 rf = pw ? static_cast<const double2*>(p.band_fyz)[r0 + r] : make_double2(1.0, 0.0);
+              const double2 f = pw ? static_cast<const double2*>(p.band_fx)[cv] : make_double2(1.0, 0.0);
+              const double2 f0 = cmul(make_double2(s * f.x, s * f.y), rf);
+              v = quiet ? cmul(v, f0) : pointwise64(v, f0, cyp);
+            }
           }
         }
       }
