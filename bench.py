@@ -161,7 +161,8 @@ def source_hash():
     import hashlib
     import re
     h = hashlib.sha256()
-    for f in ("gp_sweeps.cu", "gp_sweeps64.cu", "gp_device.cuh", "gp_internal.h", "gp_api.cu"):
+    for f in ("gp_sweeps.cu", "gp_sweeps_tile.cu", "gp_sweeps64.cu", "gp_device.cuh", "gp_split.cuh",
+              "gp_internal.h", "gp_api.cu"):
         with open(os.path.join(ROOT, "paper_1605_03958_gb300", "csrc", f)) as fh:
             code = fh.read()
         code = re.sub(r"/\*.*?\*/", " ", code, flags=re.S)
@@ -201,25 +202,27 @@ def replica_throughput(local_ms, units_per_rank, group=None, device=None):
 
 # ------------------------------------------------------------ shared helpers
 
-def sweep_kernel_names(info, prec, real):
-    """Kernel (template) names of the x, y, z sweeps a solver with gp_get_info `info` runs."""
+def sweep_kernel_names(info, prec, real, plane=False):
+    """Kernel (template) names of the x, y, z sweeps a solver with gp_get_info `info` runs
+    (plane: a 2D solve, whose y sweep sums the norm)."""
     rt = "float" if prec == "f32" else "double"
     L = info["trunc"]
     W = info["band_w"]
     c = "true" if real else "false"     # complex field
     nm = "false" if real else "true"    # the z sweep sums the norm in imaginary time only
+    ynm = nm if plane else "false"
     if info.get("line64_mask", 0) == 7:
         inc = info["inc64_mask"]
         return {"sweep_x": f"k_sweep_xinc64<{c}>" if inc & 1 else f"k_sweep_x64<{c}>",
-                "sweep_y": f"k_sweep_inc64<{c},1,false>" if inc & 2 else f"k_sweep_line64<{c},1,false>",
+                "sweep_y": f"k_sweep_inc64<{c},1,{ynm}>" if inc & 2 else f"k_sweep_line64<{c},1,false>",
                 "sweep_z": f"k_sweep_inc64<{c},2,{nm}>" if inc & 4 else f"k_sweep_line64<{c},2,{nm}>"}
     tile = info["tile_mask"]
     return {
-        "sweep_x": (f"k_sweep_x_reg<{c},{W}>" if info.get("x_reg") else
+        "sweep_x": (f"k_sweep_x_reg<{c},{W},{'true' if plane else 'false'}>" if info.get("x_reg") else
                     f"k_sweep_x_band<float,{c},{W}>" if info["band_mask"] & 1 else
                     f"k_sweep_x_stream<float,{c},{L}>" if info["fast_mask"] & 1 else f"k_sweep_x<{rt},{c}>"),
-        "sweep_y": (f"k_band_tile<{c},1,false,{W}>" if tile & 2 else
-                    f"k_sweep_band_line<float,{c},1,false,{W}>" if info["band_mask"] & 2 else
+        "sweep_y": (f"k_band_tile<{c},1,{ynm},{W}>" if tile & 2 else
+                    f"k_sweep_band_line<float,{c},1,{ynm},{W}>" if info["band_mask"] & 2 else
                     f"k_sweep_stream<float,{c},1,false,{L}>" if info["fast_mask"] & 2 else f"k_sweep_y<{rt},{c}>"),
         "sweep_z": (f"k_band_tile<{c},2,{nm},{W}>" if tile & 4 else
                     f"k_sweep_band_line<float,{c},2,{nm},{W}>" if info["band_mask"] & 4 else
@@ -611,7 +614,7 @@ def run_cuda(args):
     hbm, peak_kind = peaks()
     names = ["sweep_x", "sweep_y", "sweep_z"]
     info = s.info()
-    kernels = sweep_kernel_names(info, args.prec, real)
+    kernels = sweep_kernel_names(info, args.prec, real, NZ == 1)
     per = {}
     for i, n in enumerate(names):
         if kn[i] == 0:   # a 2D solve has no z sweep
