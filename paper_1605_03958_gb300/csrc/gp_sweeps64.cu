@@ -729,7 +729,7 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_inc64(const __grid_consta
 //   |y| from kIncY to kIncLead: q's leading term (-y, -i y) in FP64, four operations per real
 //     value and seven per complex one, the rest of e as before;
 //   |E| from kIncE to kIncBigE: E in FP64 too, nine and eighteen operations, unless the value is so
-//     small against the field's largest that two parts' error stays below 2^-10 of such an |E|'s there;
+//     small against the field's largest that two parts' error stays below 3e-17 of that;
 //   |y| > kIncLead, |E| > kIncBigE, values out of range, a tiny field: products in FP64 (they round the
 //     factors' product alike at every step: an error that grows with the steps),
 // each for a warp as a whole.
@@ -926,7 +926,7 @@ __global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_const
         Two e = factor(rc);
         const float em = fmaxf(fabsf(e.h.x), fabsf(e.h.y));
         const float size = bits_f((uint32_t)min(addmax0(vm, -kSplitOff), 253 << 20) << 3) * unit;
-        bool ok = !tiny && (em <= kIncE || (em <= kIncBigE && em * size <= 0x1p-10f));
+        bool ok = !tiny && (em <= kIncE || (em <= kIncBigE && em * size <= 0x1p-8f));
         int tmax = 0;
         float ym = 0.f;
         Two V;
