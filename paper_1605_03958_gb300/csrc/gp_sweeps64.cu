@@ -652,8 +652,10 @@ __device__ __forceinline__ void inc_segment(const IncRho<CPLX>& rho, float4* slo
   }
 }
 
+// (80 registers: six blocks of 128 threads per SM, as many as their shared memory leaves room for;
+// the z sweep with its norm took 116 by itself, and 61.9 us instead of 55.3)
 template <bool CPLX, int AXIS, bool NORM>
-__global__ void __launch_bounds__(kIncThreads) k_sweep_inc64(const __grid_constant__ SweepParams p) {
+__global__ void __maxnreg__(80) k_sweep_inc64(const __grid_constant__ SweepParams p) {
   extern __shared__ __align__(16) float4 inc_smem[];
   const int X = p.inc_x, nseg = p.inc_seg, n = p.n;
   const int tid = threadIdx.x, T = blockDim.x;
@@ -811,8 +813,10 @@ __device__ __forceinline__ double2 pointwise_lead(double2 v, Two e, const Two& V
   }
 }
 
+// (Registers, 240 x 200 x 160: real 96, 87 us, against 97 with the FP64 paths laid out freely; complex
+// 128, 197 us and 27.3 at 101 x 77 x 53; 80, 178 and 29.3)
 template <bool CPLX>
-__global__ void __launch_bounds__(kIncThreads) k_sweep_xinc64(const __grid_constant__ SweepParams p) {
+__global__ void __maxnreg__(CPLX ? 128 : 96) k_sweep_xinc64(const __grid_constant__ SweepParams p) {
   extern __shared__ __align__(16) float4 inc_smem[];
   const int X = p.inc_x, nseg = p.inc_seg, nx = p.nx;
   const int tid = threadIdx.x, T = blockDim.x, TS = T + 1;   // one slot of padding: see `place`
