@@ -436,9 +436,9 @@ __global__ void __launch_bounds__(kLineThreads) k_sweep_line64(const __grid_cons
 // formed in two-part FP32 (gp_split.cuh) and one DADD per point is left (14.7 us of FP64
 // pipe for 240 x 200 x 160 real points), against five FP64 operations per real point and
 // 18 per complex one in k_sweep_line64.  Measured at 240 x 200 x 160 (GB300, event-timed
-// launches): y 80 -> 44 us, z with its norm 106 -> 59 us; complex y 245 -> 91 us, z 290 ->
-// 83 us.  Now bound by issue (2.2-2.4 of 4 instructions per clock, 116 per real point,
-// 260 per complex one) and the FP64 pipe (34-54 %).
+// launches): y 80 -> 43 us, z with its norm 106 -> 55 us; complex y 245 -> 92 us, z 290 ->
+// 84 us.  Now bound by issue (2.1-2.3 of 4 instructions per clock, z with its norm 1.6; 113-116 per
+// real point, 252-268 per complex one) and the FP64 pipe (33-38 %, z with its norm 61 %).
 //
 // Accuracy: s is exact and the increment's 48 bits are far below the final rounding as long as
 // the increment is small against v.  Relative L2 error of a sweep against quadruple precision
@@ -736,8 +736,8 @@ __global__ void __maxnreg__(80) k_sweep_inc64(const __grid_constant__ SweepParam
 //     factors' product alike at every step: an error that grows with the steps),
 // each for a warp as a whole.
 // Measured at 240 x 200 x 160 with the solve: 284 us (k_sweep_x64 at its shortest
-// polynomial; 620 us where the density calls for the longer one) -> 92 us, complex 686
-// -> 194 us.
+// polynomial; 620 us where the density calls for the longer one) -> 87 us, complex 686
+// -> 197 us; 189 and 502 instructions per point, FP64 pipe 55 and 47 %.
 //
 // A block owns inc_x row vectors (real: pairs of rows; complex: rows) and works in three
 // passes: lanes along the rows (coalesced) for the substep, v' to the field and to the
