@@ -11,12 +11,11 @@
 // 11 at W = 5: 90 MB through L2 per sweep of a 31 MB field, and two dependent fetches.  Here
 // four runs share the halo (1.25 reads per point), all of a block's loads are in flight at
 // once, and the taps are two-lane FP32 (6.5 FP32 instructions per point instead of 12).
-// Measured per step (GB300; k_sweep_band_line -> here): 131 x 97 x 61 real 21.1 -> 16.9 us,
-// complex 21.3 -> 19.2; 300 x 256 plane 10.6 -> 8.2, complex 9.2 -> 7.4; 64 x 48 x 32 13.7 ->
-// 11.9; 240 x 200 x 160 31.9 -> 30.6, complex 66.6 -> 64.4 (since the next sweep's blocks are let
-// in at exit 131 x 97 x 61 takes 15.2 and 15.8, the plane 8.0, 240 x 200 x 160 complex 61.3).  What bounds it at 240 x 200 x 160:
-// issue and latency together (2.3 instructions per clock, 22 warps per SM); a copy of the
-// field takes 8.3 us where a sweep takes 14.
+// Measured per step (GB300; k_sweep_band_line -> here, x and y apart): 131 x 97 x 61 real 18.1 ->
+// 15.4 us, complex 17.9 -> 15.9; 300 x 256 plane 10.4 -> 8.2, complex 9.1 -> 7.6; 64 x 48 x 32 12.6 ->
+// 9.9, complex 11.0 -> 9.4; 128 x 128 x 96 16.5 -> 14.3; 240 x 200 x 160 31.4 -> 31.3.  What bounds it
+// at 240 x 200 x 160: latency and issue together (1.4-1.5 instructions per clock with cold caches, 25
+// warps per SM); a copy of the field takes 8.3 us where a sweep takes 14.
 #include <algorithm>
 #include <type_traits>
 
@@ -31,9 +30,10 @@ constexpr int kTileCols = 32;      // y / z: vector positions per block, one per
 constexpr int kTileRuns = 4;       // y / z: runs per block, one per warp
 constexpr int kBatchTileThreads = 128;   // pools: runs times columns
 constexpr int kXyThreads = 256;    // x and y together
-constexpr int kXyRows = 12;        // rows per block at most (64^3: 11.1 us a step, 15.7 with 32)
-// Grids that take it (separate -> joined, us per step, real / complex): 64^3 11.1 -> 9.2 /
-// 10.4 -> 8.9, 96 x 80 x 64 11.7 -> 10.7 / 12.1 -> 11.1, 256 x 32 x 32 10.1 -> 9.6 / 10.3 -> 9.5;
+constexpr int kXyRows = 12;        // rows per block at most (64^3 9.3 us a step, 96 x 80 x 64 complex 11.1,
+                                   // 256 x 32 x 32 9.6; with 32 rows 9.2, 12.2, 11.1)
+// Grids that take it (separate -> joined, us per step, real / complex): 64^3 11.1 -> 9.3 /
+// 10.4 -> 8.9, 96 x 80 x 64 11.7 -> 10.7 / 12.1 -> 11.1, 256 x 32 x 32 10.2 -> 9.6 / 10.3 -> 9.6;
 // and not: 131 x 97 x 61 15.4 -> 18.3 / 15.9 -> 20.0, 24 x 100 x 80 (720 blocks) 12.8 -> 13.3 /
 // 12.1 -> 11.5
 constexpr long long kXyPoints = 1 << 19, kXyBlocks = 600;
