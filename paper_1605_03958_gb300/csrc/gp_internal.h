@@ -289,7 +289,7 @@ cudaError_t launch_inc64(int axis, const SweepParams& p, bool complex_field, cud
 int stream_warps_per_sm(int axis, bool complex_field, int trunc);
 
 // Observables into p.out[0..9] (gp_obs order).  With `two` (grids for which observables_two
-// holds) by two-part FP32 sums, p.out[10] receiving the field's largest |component| and
+// holds) by sums on the FP32 pipe, p.out[10] receiving the field's largest |component| and
 // p.out[11] the pending factor: the result holds if observables_hold, else the call is
 // repeated without.
 bool observables_two(const FieldParams& p);

@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_observables(const FieldParam
   }
 }
 
-// ------------------------------------- observables in two-part FP32 sums
+// ------------------------------------- observables by sums on the FP32 pipe
 
 // The same sums with the arithmetic on the FP32 pipe (gp_split.cuh: FP64 operations and
 // conversions run at 1/64 of FP32's rate here, and k_observables spends 32-45 of them per
